@@ -12,8 +12,8 @@
 // columns.  The sweep takes 128-wide block columns j = 0, 1, ...  (right-looking):
 //   diag     the CTA of factor_diag_kernel factors the (updated) diagonal block,
 //            B_jj = L_jj L_jj^T, in shared memory and inverts it, Z_jj = L_jj^-1, into the
-//            inverse's diagonal block (32-wide tiles: one warp factors and inverts each 32 x 32
-//            tile on the diagonal, the CTA's warps update the other tiles);
+//            inverse's diagonal block (16-wide blocks: one warp factors and inverts each 16 x 16
+//            block on the diagonal and runs ahead, the CTA's other warps update the rest);
 //   strips   panel L_ij = B_ij Z_jj^T (i > j) and the inverse's row X_j,c = Z_jj R_j,c (c < j),
 //            in 64-wide strips on CUDA cores (factor_strip_kernel);
 //   updates  B_ik -= L_ij L_kj^T over the trailing square, and R_ic -= L_ij X_jc for i > j,
@@ -41,10 +41,10 @@ namespace hscale {
 namespace {
 
 constexpr int kNb = 128;                  // block of the sweep
-constexpr int kSub = 32;                  // sub-block of the diagonal factor (one warp)
+constexpr int kSub = 16;                  // sub-block of the diagonal factor (one warp)
 constexpr int kLd = kNb + 4;              // padded shared-memory row (16-byte multiple)
 constexpr int kDiagThreads = 512;
-constexpr int kDiagSmemBytes = (2 * kNb * kLd + kSub * kLd + 4 * kSub) * 4;
+constexpr int kDiagSmemBytes = (2 * kNb * kLd + 4) * 4;
 constexpr int kStripRows = 32;            // rows (or columns) of one strip
 constexpr int kStripThreads = 256;
 constexpr int kStripSmemBytes = (kNb * (kNb + 4) + kNb * (kStripRows + 4)) * 4;
@@ -136,216 +136,337 @@ __device__ __forceinline__ void record_failure(int32_t* info, int32_t order) {
   atomicCAS(reinterpret_cast<int*>(info), 0, order);
 }
 
-__device__ __forceinline__ float rsqrt_approx(float x) {
+// Fast reciprocal and reciprocal square root (relative error within about 2^-22): the quick
+// forms take operands and results in the normal range, kFull those outside it too.
+template <bool kFull>
+__device__ __forceinline__ float fast_rcp(float x) {
   float r;
-  asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  if (kFull) asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  else asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+template <bool kFull>
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float r;
+  if (kFull) asm("rsqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  else asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 
-// One warp factors the 32 x 32 block at A (row stride kLd, lower triangle) in place,
-// A = L L^T, and writes Z = L^-1 (lower, zeros above) at Zo (row stride kLd); col is a 128-float scratch (two 64-float buffers).  Lane i holds row i of
-// the block in registers (every loop has a constant trip count and every register index is a
-// constant, so the row stays in registers; kept out of line: inlined into the block kernel,
-// the compiler moves the row to local memory).  Two columns are eliminated per step: the
-// 2 x 2 pivot block gives L_jj, L_j+1,j and L_j+1,j+1, every lane scales its two entries, the
-// pairs (L_kj, L_k,j+1) go to shared memory and come back four rows per 16-byte broadcast
-// load, and each lane updates its row.  Entries above the diagonal are updated too
-// (harmlessly) and zeroed at the end.  The square roots come from the approximate hardware
-// instruction (relative error about 2^-22), which keeps the serial chain of pivots short.
-// The inverse is built in the same sweep: lane c also holds column c of Z, as partial sums
-// s_i = delta_ic - sum_{m < j} L_im Z_mc over the rows not yet final.  When columns j and
-// j + 1 of L are known, Z_jc = s_j / L_jj and Z_j+1,c = (s_j+1 - L_j+1,j Z_jc) / L_j+1,j+1
-// (forward substitution), and the later rows take s_k -= L_kj Z_jc + L_k,j+1 Z_j+1,c with
-// the same broadcast loads as the factor's update, so no second serial pass is needed.
-// Each step updates the next pivot pair's two rows first and computes that pair's pivots
-// before the rest of its update, so the serial chain of the next step can run alongside this
-// step's bulk of independent FMAs; the pivot columns alternate between the two scratch
-// buffers, so one __syncwarp per step orders them.  A pivot that is not positive is kept in a
-// register (the first one) and recorded once at the end, so no step branches.  Every value
-// takes the same operations in the same order as a plain right-looking sweep.
-
-// The pivot pair (j, j + 1) from the current rows (the 2 x 2 block comes from lanes j and
-// j + 1): this lane's entries v0 = L_lane,j and v1 = L_lane,j+1 (zero above the diagonal),
-// rows j and j + 1 of Z in this lane's column (1 / L_jj = ra, 1 / L_j+1,j+1 = rc), all four
-// written back into r and z.
-__device__ __forceinline__ void pivot_pair(float (&r)[kSub], float (&z)[kSub], const int j, int lane,
-                                           int32_t base, int32_t& fail, float& v0, float& v1, float& zj,
-                                           float& zj1) {
+// One warp factors the 16 x 16 block at A (row stride kLd, lower triangle), A = L L^T, and
+// writes Z = L^-1 (lower, zeros above) at Zo (row stride kLd).  The block's own L is not
+// needed: only Z is written.
+//
+// Two halves of the warp run the same instructions: lane i < 16 holds row i of the block,
+// lane 16 + c holds column c of the unit-lower inverse Y, which starts as the identity.  The
+// elimination is A = M diag(d) M^T with unit-lower M, two pivots per step: with the pivot
+// columns C0 (column j) and C1' = C1 - C0 b / a (column j + 1 after pivot j), every lane forms
+// its x0 = r_j / a and x1 = r'_j+1 / d_j+1 and subtracts C0_k x0 + C1'_k x1 from its entry k:
+// for a row this is the Schur update, for a column of Y the forward substitution, and
+// both take the same pair (C0_k, C1'_k), by shuffle from lane k.  At the end row i of Y is
+// scaled by 1 / sqrt(d_i), which gives Z.
+//
+// What bounds it is the chain from one pivot pair to the next, so that chain
+// holds no square root, and its two reciprocals run side by side: 1 / a, and 1 / det of the
+// 2 x 2 pivot block (1 / d_j+1 = a / det).  Each step forms the next pivot block first, the same
+// in every lane from entries shuffled before the update (no shuffle of updated values on the
+// chain), and the rest of its update fits in the chain's shadow.  The reciprocals are
+// the approximate hardware ones.  A pivot that is not positive is kept in a register (the first
+// one) and recorded once at the end, so no step branches.
+//
+// Measured on one GB300: 1.7 K cycles per 16 columns beside the other warps' products; the
+// 32-wide sweep before this one, a Cholesky with square roots on the chain and 64 values per
+// lane, took 7.5 K per 32 columns.
+//
+// Returns whether every pivot was in the range of the quick reciprocals (if not, nothing was
+// recorded and Zo is to be formed again with kFull).
+template <bool kFull>
+__device__ __forceinline__ bool factor_sub16(const float* A, float* Zo, int lane, int32_t* info, int32_t base) {
   const unsigned full = 0xFFFFFFFFu;
-  float a = __shfl_sync(full, r[j], j);
-  const float b = __shfl_sync(full, r[j], j + 1);
-  const float c = __shfl_sync(full, r[j + 1], j + 1);
-  const bool bad_a = !(a > 0.0f);
-  fail = (fail == 0 && bad_a) ? base + j + 1 : fail;
-  a = bad_a ? 1.0f : a;
-  const float ra = rsqrt_approx(a);
-  const float l00 = __fmul_rn(a, ra), l10 = __fmul_rn(b, ra);
-  float c2 = __fmaf_rn(-l10, l10, c);
-  const bool bad_c = !(c2 > 0.0f);
-  fail = (fail == 0 && bad_c) ? base + j + 2 : fail;
-  c2 = bad_c ? 1.0f : c2;
-  const float rc = rsqrt_approx(c2);
-  const float l11 = __fmul_rn(c2, rc);
-  const float x0 = __fmul_rn(r[j], ra);
-  const float x1 = __fmul_rn(__fmaf_rn(-x0, l10, r[j + 1]), rc);
-  v0 = lane == j ? l00 : (lane == j + 1 ? l10 : (lane > j + 1 ? x0 : 0.0f));
-  v1 = lane == j + 1 ? l11 : (lane > j + 1 ? x1 : 0.0f);
-  r[j] = v0;
-  r[j + 1] = v1;
-  zj = __fmul_rn(z[j], ra);
-  zj1 = __fmul_rn(__fmaf_rn(-l10, zj, z[j + 1]), rc);
-  z[j] = zj;
-  z[j + 1] = zj1;
-}
-
-// Rows k and k + 1 of this lane's row and Z column take the pivot pair's update; cb holds
-// the pairs (L_kj, L_k,j+1) of every row.
-__device__ __forceinline__ void update_pair(float (&r)[kSub], float (&z)[kSub], const int k, const float* cb,
-                                            float v0, float v1, float zj, float zj1) {
-  const float4 q = *reinterpret_cast<const float4*>(cb + 2 * k);  // (L_kj, L_k,j+1, L_k+1,j, L_k+1,j+1)
-  r[k] = __fmaf_rn(-v0, q.x, __fmaf_rn(-v1, q.y, r[k]));
-  r[k + 1] = __fmaf_rn(-v0, q.z, __fmaf_rn(-v1, q.w, r[k + 1]));
-  z[k] = __fmaf_rn(-q.x, zj, __fmaf_rn(-q.y, zj1, z[k]));
-  z[k + 1] = __fmaf_rn(-q.z, zj, __fmaf_rn(-q.w, zj1, z[k + 1]));
-}
-
-__device__ __noinline__ void factor_sub32(float* A, float* Zo, float* col, int lane, int32_t* info,
-                                          int32_t base) {
-  float r[kSub], z[kSub];
+  const bool is_row = lane < kSub;
+  const int li = lane & (kSub - 1);
+  float r[kSub], zs[kSub];  // the row or column; 1 / sqrt(d_k)
 #pragma unroll
   for (int k = 0; k < kSub; k += 4) {
-    const float4 a = *reinterpret_cast<const float4*>(A + lane * kLd + k);
-    r[k] = a.x;
-    r[k + 1] = a.y;
-    r[k + 2] = a.z;
-    r[k + 3] = a.w;
+    const float4 a = *reinterpret_cast<const float4*>(A + li * kLd + k);
+    r[k] = is_row ? a.x : (k == li ? 1.0f : 0.0f);
+    r[k + 1] = is_row ? a.y : (k + 1 == li ? 1.0f : 0.0f);
+    r[k + 2] = is_row ? a.z : (k + 2 == li ? 1.0f : 0.0f);
+    r[k + 3] = is_row ? a.w : (k + 3 == li ? 1.0f : 0.0f);
   }
-#pragma unroll
-  for (int k = 0; k < kSub; ++k) z[k] = k == lane ? 1.0f : 0.0f;
   int32_t fail = 0;
-  float v0, v1, zj, zj1;
-  pivot_pair(r, z, 0, lane, base, fail, v0, v1, zj, zj1);
+  float lo = 1.0f, hi = 1.0f;  // the range of the pivots
+  float ia, ic, r1;
+  // the pivots j and j + 1 from the pivot block [a b; b c] (the same in every lane): ia = 1 / d_j,
+  // ic = 1 / d_j+1, r1 = this lane's entry j + 1 after pivot j
+  auto pivot = [&](int j, float a, float b, float c) {
+    const bool bad_a = !(a > 0.0f);
+    fail = (fail == 0 && bad_a) ? base + j + 1 : fail;
+    a = bad_a ? 1.0f : a;
+    ia = fast_rcp<kFull>(a);
+    const float m = __fmul_rn(b, ia);
+    // det 2^-e, e the exponent of a, so that it has the magnitude of d_j+1 = det / a
+    const float as = __uint_as_float((__float_as_uint(a) & 0x007FFFFFu) | 0x3F800000u);  // a 2^-e
+    const float bs = __fmul_rn(b, __uint_as_float(0x7F000000u - (__float_as_uint(a) & 0x7F800000u)));
+    float det = __fmaf_rn(as, c, -__fmul_rn(bs, b));
+    if (kFull) det = __fmul_rn(as, __fmaf_rn(-m, b, c));
+    const bool bad_c = !(det > 0.0f);
+    fail = (fail == 0 && bad_c) ? base + j + 2 : fail;
+    det = bad_c ? as : det;
+    ic = __fmul_rn(as, fast_rcp<kFull>(det));
+    r1 = __fmaf_rn(-m, r[j], r[j + 1]);
+    lo = fminf(lo, fminf(a, det));
+    hi = fmaxf(hi, fmaxf(a, det));
+  };
+  pivot(0, __shfl_sync(full, r[0], 0), __shfl_sync(full, r[0], 1), __shfl_sync(full, r[1], 1));
 #pragma unroll
-  for (int j = 0; j + 2 < kSub; j += 2) {
-    float* cb = col + ((j >> 1) & 1) * (2 * kSub);
-    reinterpret_cast<float2*>(cb)[lane] = make_float2(v0, v1);
-    __syncwarp();
-    update_pair(r, z, j + 2, cb, v0, v1, zj, zj1);
-    float n0, n1, nz0, nz1;
-    pivot_pair(r, z, j + 2, lane, base, fail, n0, n1, nz0, nz1);
+  for (int j = 0; j < kSub; j += 2) {
+    const float rj = r[j], rj1 = r1, ja = ia, jc = ic;
+    r[j + 1] = r1;
+    const float x0 = __fmul_rn(rj, ja), x1 = __fmul_rn(rj1, jc);
+    if (j + 2 < kSub) {
+      // the next pivot block before this step's update, and the pivot columns' entries in its
+      // two rows: every lane forms the updated block itself, the same way lanes j + 2 and j + 3
+      // update their rows
+      const int k = j + 2;
+      const float a0 = __shfl_sync(full, r[k], k), b0 = __shfl_sync(full, r[k], k + 1);
+      const float c0 = __shfl_sync(full, r[k + 1], k + 1);
+      const float s0 = __shfl_sync(full, rj, k), t0 = __shfl_sync(full, rj, k + 1);
+      const float s1 = __shfl_sync(full, rj1, k), t1 = __shfl_sync(full, rj1, k + 1);
+      const float u0 = __fmul_rn(s0, ja), v0 = __fmul_rn(t0, ja), u1 = __fmul_rn(s1, jc), v1 = __fmul_rn(t1, jc);
+      r[k] = __fmaf_rn(-s1, x1, __fmaf_rn(-s0, x0, r[k]));
+      r[k + 1] = __fmaf_rn(-t1, x1, __fmaf_rn(-t0, x0, r[k + 1]));
+      pivot(k, __fmaf_rn(-s1, u1, __fmaf_rn(-s0, u0, a0)), __fmaf_rn(-s1, v1, __fmaf_rn(-s0, v0, b0)),
+            __fmaf_rn(-t1, v1, __fmaf_rn(-t0, v0, c0)));
 #pragma unroll
-    for (int k = j + 4; k < kSub; k += 2) update_pair(r, z, k, cb, v0, v1, zj, zj1);
-    v0 = n0;
-    v1 = n1;
-    zj = nz0;
-    zj1 = nz1;
+      for (int i = j + 4; i < kSub; ++i)
+        r[i] = __fmaf_rn(-__shfl_sync(full, rj1, i), x1, __fmaf_rn(-__shfl_sync(full, rj, i), x0, r[i]));
+    }
+    zs[j] = __fmul_rn(ja, fast_rsqrt<kFull>(ja));
+    zs[j + 1] = __fmul_rn(jc, fast_rsqrt<kFull>(jc));
   }
+  if (!kFull && !(lo >= 0x1p-100f && hi <= 0x1p100f)) return false;
   if (fail != 0 && lane == 0) record_failure(info, fail);
+  // lane 16 + c holds column c of Y: row i is zero above the diagonal (i < c)
+  if (!is_row) {
 #pragma unroll
-  for (int k = 0; k < kSub; k += 4)
-    *reinterpret_cast<float4*>(A + lane * kLd + k) =
-        make_float4(k <= lane ? r[k] : 0.0f, k + 1 <= lane ? r[k + 1] : 0.0f, k + 2 <= lane ? r[k + 2] : 0.0f,
-                    k + 3 <= lane ? r[k + 3] : 0.0f);
-  // lane c holds column c of Z: row i is zero above the diagonal (i < c)
-#pragma unroll
-  for (int i = 0; i < kSub; ++i) Zo[i * kLd + lane] = i >= lane ? z[i] : 0.0f;
+    for (int i = 0; i < kSub; ++i) Zo[i * kLd + li] = i >= li ? __fmul_rn(r[i], zs[i]) : 0.0f;
+  }
+  __syncwarp();
+  return true;
+}
+__device__ __noinline__ void factor_sub16_full(const float* A, float* Zo, int lane, int32_t* info, int32_t base) {
+  factor_sub16<true>(A, Zo, lane, info, base);
 }
 
-// Warp-tile products on 32 x 32 tiles in shared memory (row stride kLd = 4 mod 32 words, a
-// multiple of 4).  A warp computes 16 rows of the output tile: lane (h = lane / 16,
-// cl = lane % 16) holds rows h + 2 r (r < 8) and columns cl, cl + 16 in acc[r][0..1]
-// (independent accumulators).  Per four m, A's rows are read as 16-byte words (two rows per
-// warp, four banks apart: one wavefront), and B either row by row (kNT false: B[m][c] at
-// B + m kLd + c; consecutive lanes, consecutive words) or, for a transposed operand, in place
-// from its rows (kNT true: B[m][c] at B + c kLd + m; lanes cl read rows cl and cl + 16 as
-// 16-byte words, four banks apart: two wavefronts each), so no transposed copy is needed.
-//   acc[r][q] += sum_m A[h + 2 r][m] B[m][cl + 16 q]   (-= with kNeg), over m in order
-template <bool kNT, bool kNeg = false>
-__device__ __forceinline__ void tile_mma(float (&acc)[8][2], const float* A, const float* B, int lane) {
-  const int h = lane >> 4, cl = lane & 15;
-#pragma unroll 2
+// One warp's product of 16 x 16 blocks in shared memory (row stride kLd = 4 mod 32 words).
+// A lane holds rows h, h + 8 and four columns: 4 cl + q (kNT false) or cl + 4 q (kNT true).
+// Per four m, A's rows are 16-byte words, and B is read either row by row (kNT false: B[m][c]
+// at B + m kLd + c) or in place from the transposed operand's rows (kNT true: B[m][c] at
+// B + c kLd + m), 16-byte words too.  Shared-memory reads bound these products (a 16-byte read
+// takes four cycles of the SM, two when neighbouring lanes i and i ^ 1, or i and i ^ 2, share
+// the address; measured), so h leaves out lane bit 0, cl lane bit 1, and the rows and columns
+// are dealt so that no read or write meets a bank twice.
+//   acc[r][q] += sum_m A[h + 8 r][m] B[m][column q]   (-= with kNeg), over m in order
+__device__ __forceinline__ int block_row(int lane) { return ((lane >> 3) & 3) + 2 * (lane & 2); }
+__device__ __forceinline__ int block_col(int lane) { return ((lane >> 1) & 2) + (lane & 1); }
+
+template <bool kNT, bool kNeg>
+__device__ __forceinline__ void block_mma(float (&acc)[2][4], const float* A, const float* B, int lane) {
+  const int h = block_row(lane), cl = block_col(lane);
+#pragma unroll
   for (int m = 0; m < kSub; m += 4) {
-    float b[4][2];
+    float b[4][4];  // b[m][q]
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 v = kNT ? *reinterpret_cast<const float4*>(B + (cl + 4 * q) * kLd + m)
+                           : *reinterpret_cast<const float4*>(B + (m + q) * kLd + 4 * cl);
+      const float e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) (kNT ? b[k][q] : b[q][k]) = kNeg ? -e[k] : e[k];
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const float4 v = *reinterpret_cast<const float4*>(A + (h + 8 * r) * kLd + m);
+      const float a[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = __fmaf_rn(a[k], b[k][q], acc[r][q]);
+    }
+  }
+}
+__device__ __forceinline__ void block_zero(float (&acc)[2][4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) acc[0][q] = acc[1][q] = 0.0f;
+}
+template <bool kNT>
+__device__ __forceinline__ void block_load(float (&acc)[2][4], const float* T, int lane) {
+  const int h = block_row(lane), cl = block_col(lane);
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[r][q] = T[(h + 8 * r) * kLd + (kNT ? cl + 4 * q : 4 * cl + q)];
+}
+template <bool kNT>
+__device__ __forceinline__ void block_store(const float (&acc)[2][4], float* T, int lane) {
+  const int h = block_row(lane), cl = block_col(lane);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
     if (kNT) {
-      const float4 u = *reinterpret_cast<const float4*>(B + cl * kLd + m);
-      const float4 v = *reinterpret_cast<const float4*>(B + (cl + 16) * kLd + m);
-      b[0][0] = u.x; b[1][0] = u.y; b[2][0] = u.z; b[3][0] = u.w;
-      b[0][1] = v.x; b[1][1] = v.y; b[2][1] = v.z; b[3][1] = v.w;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) T[(h + 8 * r) * kLd + cl + 4 * q] = acc[r][q];
     } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        b[q][0] = B[(m + q) * kLd + cl];
-        b[q][1] = B[(m + q) * kLd + cl + 16];
-      }
+      *reinterpret_cast<float4*>(T + (h + 8 * r) * kLd + 4 * cl) =
+          make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
     }
-    if (kNeg) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        b[q][0] = -b[q][0];
-        b[q][1] = -b[q][1];
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const float4 a = *reinterpret_cast<const float4*>(A + (h + 2 * r) * kLd + m);
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        acc[r][q] = __fmaf_rn(a.x, b[0][q], acc[r][q]);
-        acc[r][q] = __fmaf_rn(a.y, b[1][q], acc[r][q]);
-        acc[r][q] = __fmaf_rn(a.z, b[2][q], acc[r][q]);
-        acc[r][q] = __fmaf_rn(a.w, b[3][q], acc[r][q]);
-      }
-    }
-  }
-}
-__device__ __forceinline__ void tile_zero(float (&acc)[8][2]) {
-#pragma unroll
-  for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = 0.0f;
-}
-__device__ __forceinline__ void tile_load(float (&acc)[8][2], const float* T, int lane) {
-  const int h = lane >> 4, cl = lane & 15;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    acc[r][0] = T[(h + 2 * r) * kLd + cl];
-    acc[r][1] = T[(h + 2 * r) * kLd + cl + 16];
-  }
-}
-__device__ __forceinline__ void tile_store(const float (&acc)[8][2], float* T, int lane, float sign) {
-  const int h = lane >> 4, cl = lane & 15;
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    T[(h + 2 * r) * kLd + cl] = sign * acc[r][0];
-    T[(h + 2 * r) * kLd + cl + 16] = sign * acc[r][1];
   }
 }
 
-constexpr int kHalf = kSub / 2;           // rows of a tile per warp (two warps per tile)
+// The same for a 16 x 32 tile, C -= A B^T: a lane holds rows 2 h, 2 h + 1, 2 h + 8,
+// 2 h + 9 and columns cl + 8 q (q < 4), which reads 32 bytes of shared memory per 16 products instead of 48.
+__device__ __forceinline__ void wide_sub_nt(float* C, const float* A, const float* B, int lane) {
+  const int h2 = (lane & 2) + ((lane >> 2) & 4), cl = (lane & 1) + ((lane >> 1) & 2) + ((lane >> 1) & 4);
+  constexpr int kRow[4] = {0, 1, 8, 9};
+  float acc[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[r][q] = C[(h2 + kRow[r]) * kLd + cl + 8 * q];
+#pragma unroll
+  for (int m = 0; m < kSub; m += 4) {
+    float4 b[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const float4*>(B + (cl + 8 * q) * kLd + m);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float4 a = *reinterpret_cast<const float4*>(A + (h2 + kRow[r]) * kLd + m);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        acc[r][q] = __fmaf_rn(-a.x, b[q].x, acc[r][q]);
+        acc[r][q] = __fmaf_rn(-a.y, b[q].y, acc[r][q]);
+        acc[r][q] = __fmaf_rn(-a.z, b[q].z, acc[r][q]);
+        acc[r][q] = __fmaf_rn(-a.w, b[q].w, acc[r][q]);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) C[(h2 + kRow[r]) * kLd + cl + 8 * q] = acc[r][q];
+}
 
-// Factor the 128 x 128 diagonal block at (j0, j0) of Bw and invert the factor: Z_jj = L_jj^-1
-// into Xw's diagonal block (zeros above the diagonal).  The block is a 4 x 4 grid of 32 x 32
-// tiles, taken in tile columns p = 0..3:
-//   (a) warp 0 factors the tile on the diagonal and inverts it (factor_sub32);
-//   (b) the tiles below it: L_ip = B_ip Z_p^T, two warps per tile;
-//   (c) the tiles of the rest of the block: B_ik -= L_ip L_kp^T, two warps per tile (at most
-//       six tiles: one round of the sixteen warps).
-// Z_p^T and L_kp^T are read in place (the transposed form of the tile product).  The inverse
-// of the block is built by tile rows q = 1..3, X_qr = -Z_q T_qr with
-// T_qr = sum_{m=r}^{q-1} L_qm X_mr (r < q), on six warps while warp 0 runs (a): T_qr needs
-// only the tile columns m < q, and X_qr only Z_q besides, so during (a) of step p they form
-// row p - 1 (its X) and then row p (its T); row 3's X follows the sweep.  Those six warps
-// (2, 3, 6, 7, 10, 11) sit on the two schedulers that warp 0 does not use: sharing warp 0's
-// scheduler, they slowed its serial sweep (n = 4096: 1.69 against 1.65 ms).
+// Factor the 128 x 128 block in S (row stride kLd, lower triangle; B_jj = L_jj L_jj^T) and
+// invert the factor: Z_jj = L_jj^-1 in X (zero on entry above the diagonal; lower).  The block
+// is an 8 x 8 grid of 16 x 16 blocks, taken in columns p = 0..7:
+//   (a) warp 0 factors and inverts the block on the diagonal (factor_sub16): Z_p into X_pp;
+//   (b) one warp each: the blocks below it, L_ip = B_ip Z_p^T (i > p, in place), and the
+//       inverse's row, X_pc = Z_p T_pc (c < p, in place);
+//   (c) right-looking in S, B_ik -= L_ip L_kp^T (p < k <= i), and left-looking in X, the next
+//       row's T_p+1,c = -sum_{k=c..p} L_p+1,k X_kc (c <= p).
+// Warp 0 runs ahead: of (b) and (c) it takes only the products on the way to the next diagonal
+// block, L_p+1,p and B_p+1,p+1, and goes on to its (a) while the other warps run the rest,
+// taking the products of (c) one at a time from a counter (the longest sums first).  A column
+// costs the slower of the two.  Left-looking in X keeps (c) even: 19 to 28 products in every
+// column, where right-looking would put 34 in the first and 7 in the last.
+// Bound by the reads of shared memory in (c) (16 bytes a lane take two to four cycles of the SM)
+// and, behind them, by the sub-factors.  One GB300: 29 K cycles per 128-block, against 52 K for
+// 32-wide tiles without look-ahead; n = 4096: the call 1755 -> 1540 us.
+constexpr int kGrid16 = kNb / kSub;
+__device__ __forceinline__ void factor_block128(float* S, float* X, int* next, int tid, int32_t* info, int32_t j0) {
+  const int lane = tid & 31, warp = tid >> 5;
+  auto sub = [&](float* A, float* Z, int32_t base) {
+    if (!factor_sub16<false>(A, Z, lane, info, base)) factor_sub16_full(A, Z, lane, info, base);
+  };
+  if (warp == 0) sub(S, X, j0);
+  __syncthreads();
+  for (int p = 0; p < kGrid16; ++p) {
+    const int c0 = p * kSub, d0 = c0 + kSub;
+    const float* Zp = X + c0 * kLd + c0;
+    auto panel = [&](int i) {
+      float* P = S + i * kSub * kLd + c0;
+      float acc[2][4];
+      block_zero(acc);
+      block_mma<true, false>(acc, P, Zp, lane);
+      __syncwarp();
+      block_store<true>(acc, P, lane);
+    };
+    if (warp == 0) {
+      if (p + 1 == kGrid16) break;
+      panel(p + 1);
+      __syncwarp();
+      asm volatile("bar.arrive 1, 512;" ::: "memory");  // L_p+1,p is in place
+      float acc[2][4];
+      float* D = S + d0 * kLd + d0;
+      block_load<true>(acc, D, lane);
+      block_mma<true, true>(acc, S + d0 * kLd + c0, S + d0 * kLd + c0, lane);
+      block_store<true>(acc, D, lane);
+      __syncwarp();
+      sub(D, X + d0 * kLd + d0, j0 + d0);
+    } else {
+      // (b): c < p on warps 1..p, i > p + 1 on warps p + 1..6 (7 in the last column)
+      if (warp <= p) {
+        float* T = X + c0 * kLd + (warp - 1) * kSub;
+        float acc[2][4];
+        block_zero(acc);
+        block_mma<false, false>(acc, Zp, T, lane);
+        __syncwarp();
+        block_store<false>(acc, T, lane);
+      } else if (warp + 1 < kGrid16) {
+        panel(warp + 1);
+      } else if (tid == kDiagThreads - 1) {
+        *next = 0;
+      }
+      if (p + 1 == kGrid16) break;
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      // (c): T_p+1,c for c = 0..p, then rows i > p + 1 of S, two blocks (i, k), (i, k + 1)
+      // at a time
+      for (;;) {
+        int e = 0;
+        if (lane == 0) e = atomicAdd(next, 1);
+        e = __shfl_sync(0xFFFFFFFFu, e, 0);
+        if (e <= p) {
+          float acc[2][4];
+          block_zero(acc);
+          for (int k = e; k <= p; ++k)
+            block_mma<false, true>(acc, S + d0 * kLd + k * kSub, X + k * kSub * kLd + e * kSub, lane);
+          block_store<false>(acc, X + d0 * kLd + e * kSub, lane);
+          continue;
+        }
+        int i = p + 2, k = e - (p + 1);  // row i has (i - p + 1) / 2 tiles
+        while (i < kGrid16 && k >= (i - p + 1) / 2) {
+          k -= (i - p + 1) / 2;
+          ++i;
+        }
+        if (i >= kGrid16) break;
+        k = p + 1 + 2 * k;
+        float* C = S + i * kSub * kLd + k * kSub;
+        const float* L = S + i * kSub * kLd + c0;
+        if (k < i) {
+          wide_sub_nt(C, L, S + k * kSub * kLd + c0, lane);
+        } else {
+          float acc[2][4];
+          block_load<true>(acc, C, lane);
+          block_mma<true, true>(acc, L, L, lane);
+          block_store<true>(acc, C, lane);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+}
+
+// The diagonal block at (j0, j0) of Bw: Z_jj into Xw's diagonal block (zeros above the
+// diagonal).  One CTA.  Only the lower triangle of the block is used.
 __global__ void __launch_bounds__(kDiagThreads, 1)
 factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* __restrict__ Xw,
                    int32_t* __restrict__ info) {
   extern __shared__ __align__(16) float sm[];
   float* S = sm;                 // [128][kLd] the block, then L (lower)
   float* X = S + kNb * kLd;      // [128][kLd] the inverse (lower)
-  float* T = X + kNb * kLd;      // [32][kLd] the T tiles of the inverse's current row
-  float* col = T + kSub * kLd;   // [128] the pivot columns of factor_sub32
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int h0 = kHalf * (warp & 1);  // the first of a warp's 16 rows within its tile
-  const int pair = warp >> 1;         // which tile a warp works on (of up to eight at a time)
+  int* next = reinterpret_cast<int*>(X + kNb * kLd);  // the counter of factor_block128
+  const int tid = threadIdx.x;
 
   // programmatic dependent launch: the strips may be scheduled now; the previous step's update
   // must have finished before the block is read
@@ -353,7 +474,7 @@ factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* 
   pdl_wait_primary();
   const float* blk = Bw + j0 * ld + j0;
   // independent 16-byte loads per thread in flight
-#pragma unroll 4
+#pragma unroll
   for (int t = 0; t < kNb * kNb / 4 / kDiagThreads; ++t) {
     const int e = tid + t * kDiagThreads;
     const int r = e >> 5, c = (e & 31) * 4;
@@ -361,75 +482,7 @@ factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* 
     *reinterpret_cast<float4*>(X + r * kLd + c) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __syncthreads();
-
-  for (int p = 0; p < kNb / kSub; ++p) {
-    const int c0 = p * kSub;
-    if (warp == 0) {
-      factor_sub32(S + c0 * kLd + c0, X + c0 * kLd + c0, col, lane, info, (int32_t)(j0 + c0));
-    } else if ((warp & 2) != 0 && warp < 12 && p >= 1) {
-      // warps 2, 3, 6, 7, 10, 11: the schedulers that warp 0 does not use
-      const int u = warp >> 2;        // the tile column r = u of the inverse's row
-      if (p >= 2) {
-        // X_qr = -Z_q T_qr for q = p - 1
-        const int q0 = (p - 1) * kSub;
-        if (u < p - 1) {
-          float acc[8][2];
-          tile_zero(acc);
-          tile_mma<false>(acc, X + (q0 + h0) * kLd + q0, T + u * kSub, lane);
-          tile_store(acc, X + (q0 + h0) * kLd + u * kSub, lane, -1.0f);
-        }
-        asm volatile("bar.sync 1, 192;" ::: "memory");  // these six warps: X_q done, T tiles free
-      }
-      // T_pr = sum_{m=r}^{p-1} L_pm X_mr
-      if (u < p) {
-        float acc[8][2];
-        tile_zero(acc);
-        for (int m = u; m < p; ++m)
-          tile_mma<false>(acc, S + (c0 + h0) * kLd + m * kSub, X + m * kSub * kLd + u * kSub, lane);
-        tile_store(acc, T + h0 * kLd + u * kSub, lane, 1.0f);
-      }
-    }
-    __syncthreads();
-    // (b) tiles below: L_ip = B_ip Z_p^T
-    const int below = kNb / kSub - 1 - p;
-    if (below == 0) break;
-    if (pair < below) {
-      const int r0 = c0 + kSub * (1 + pair) + h0;  // this warp's first row
-      float acc[8][2];
-      tile_zero(acc);
-      tile_mma<true>(acc, S + r0 * kLd + c0, X + c0 * kLd + c0, lane);
-      __syncwarp();
-      tile_store(acc, S + r0 * kLd + c0, lane, 1.0f);
-    }
-    __syncthreads();
-    // (c) tiles (i, k), p < k <= i: B_ik -= L_ip L_kp^T
-    {
-      int t = pair, i = p + 1;
-      while (i < kNb / kSub && t > i - (p + 1)) {
-        t -= i - p;
-        ++i;
-      }
-      if (i < kNb / kSub) {
-        const int k0 = (p + 1 + t) * kSub, r0 = i * kSub + h0;
-        float acc[8][2];
-        tile_load(acc, S + r0 * kLd + k0, lane);
-        tile_mma<true, true>(acc, S + r0 * kLd + c0, S + k0 * kLd + c0, lane);
-        tile_store(acc, S + r0 * kLd + k0, lane, 1.0f);
-      }
-    }
-    __syncthreads();
-  }
-
-  // the inverse's last tile row: X_3r = -Z_3 T_3r
-  if (pair < kNb / kSub - 1) {
-    const int q0 = kNb - kSub;
-    float acc[8][2];
-    tile_zero(acc);
-    tile_mma<false>(acc, X + (q0 + h0) * kLd + q0, T + pair * kSub, lane);
-    tile_store(acc, X + (q0 + h0) * kLd + pair * kSub, lane, -1.0f);
-  }
-  __syncthreads();
-
+  factor_block128(S, X, next, tid, info, (int32_t)j0);
   // write-out: Z into Xw's diagonal block (16-byte words).  L_jj itself is not needed again:
   // the panel uses Z_jj, and the rest of the sweep reads only the blocks below the diagonal.
   float* xo = Xw + j0 * ld + j0;
