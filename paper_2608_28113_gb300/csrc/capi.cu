@@ -73,11 +73,12 @@ int hscale_abi_version(void) { return 4; }
 
 int hscale_device_error_flags(uint32_t* flags) {
   if (flags == nullptr) return HSCALE_ERR_NULL;
-  uint32_t a = 0, b = 0, c = 0;
+  uint32_t a = 0, b = 0, c = 0, d = 0;
   cudaError_t err = hscale::read_hessian_device_error(&a);
   if (err == cudaSuccess) err = hscale::read_output_error_device_error(&b);
   if (err == cudaSuccess) err = hscale::read_selftest_device_error(&c);
-  *flags = a | b | c;
+  if (err == cudaSuccess) err = hscale::read_update_device_error(&d);
+  *flags = a | b | c | d;
   return from_cuda(err);
 }
 
@@ -326,7 +327,7 @@ inline int64_t round256(int64_t bytes) { return (bytes + 255) / 256 * 256; }
 }  // namespace
 
 // running weights (fp32 m x n) and two buffers each of the bf16 split operands of the
-// update GEMM: A' (m x 6 block) and B' (n x 6 block)
+// update: E (m x 3 block, in regions of m x 6 block) and U's rows (n x 3 block, likewise)
 size_t hscale_gptq_workspace_bytes(int64_t m, int64_t n, int32_t block) {
   if (m <= 0 || n <= 0 || block <= 0) return 0;
   const int64_t b = block;
@@ -351,10 +352,10 @@ int hscale_gptq_hscale(const void* w_bf16, int64_t m, int64_t n, const float* U,
   uint8_t* base = static_cast<uint8_t*>(workspace);
   const int64_t b = block;
   float* Wf = reinterpret_cast<float*>(base);
-  uint16_t* A6 = reinterpret_cast<uint16_t*>(base + round256(m * n * 4));
-  uint16_t* B6 = reinterpret_cast<uint16_t*>(base + round256(m * n * 4) + round256(2 * m * 6 * b * 2));
+  uint16_t* Es = reinterpret_cast<uint16_t*>(base + round256(m * n * 4));
+  uint16_t* Us = reinterpret_cast<uint16_t*>(base + round256(m * n * 4) + round256(2 * m * 6 * b * 2));
   return from_cuda(hscale::launch_gptq_hscale(w_bf16, m, n, U, h, global_scale, dead, block, down, up, codes_out,
-                                              packed_out, Wf, A6, B6, as_stream(stream)));
+                                              packed_out, Wf, Es, Us, as_stream(stream)));
 }
 
 int hscale_pack_nvfp4(const void* w_bf16, int64_t m, int64_t n, const float* global_scale,

@@ -17,6 +17,7 @@
 
 #include "hscale_device.cuh"
 #include "hscale_internal.h"
+#include "split3.cuh"
 
 namespace hscale {
 namespace {
@@ -48,29 +49,11 @@ __device__ float exact_group_score(const float (&a)[16], const float (&hj)[16], 
   return t[0];
 }
 
-// The update W[:, c1:] -= E U[col0:c1, c1:] (c1 = col0 + B) runs on the tensor cores with
-// fp32-level accuracy: every fp32 value x is split into three bf16 parts x1 + x2 + x3 (each
-// difference exact in fp32, so the parts carry x to about 2^-24 relative), and the six
-// products E1 U1, E1 U2, E2 U1, E1 U3, E2 U2, E3 U1 (every pair whose weight is above
-// 2^-24) are one bf16 GEMM over K = 6B with fp32 accumulation: A' = [-E1 | -E1 | -E2 | -E1
-// | -E2 | -E3] against B' = [U1 | U2 | U1 | U3 | U2 | U1] (the negation makes the GEMM's
-// accumulate a subtract).
-__device__ __forceinline__ void split3(float x, uint16_t (&p)[3]) {
-  const __nv_bfloat16 a = __float2bfloat16_rn(x);
-  const float r1 = __fsub_rn(x, __bfloat162float(a));
-  const __nv_bfloat16 b = __float2bfloat16_rn(r1);
-  const float r2 = __fsub_rn(r1, __bfloat162float(b));
-  const __nv_bfloat16 c = __float2bfloat16_rn(r2);
-  p[0] = __bfloat16_as_ushort(a);
-  p[1] = __bfloat16_as_ushort(b);
-  p[2] = __bfloat16_as_ushort(c);
-}
-
 // Four lanes (a quad) per group: each scores every fourth candidate of the window with exact
 // decisions, the quad keeps the best under the search's tie rule (a total order, so every
 // lane ends with the same code), and each lane writes the nibbles of four of the group's
-// elements and their scaled errors E = (w - w_hat) / U_jj, split, into the update's A
-// operand [m, 6B]: A' = [-E1 | -E1 | -E2 | -E1 | -E2 | -E3], four bf16 (8 bytes) per segment.
+// elements and their scaled errors E = (w - w_hat) / U_jj, split in three bf16 parts, into the
+// update's operand [m, 3 B] (update.cu), four bf16 (8 bytes) per part.
 __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W, int64_t m, int64_t n, int64_t col0,
                                                     int B, const float* __restrict__ h, const float* __restrict__ U,
                                                     const float* __restrict__ global_scale, int down, int up,
@@ -129,7 +112,7 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
     const float4 wq = reinterpret_cast<const float4*>(W + r * n + col)[q];
     const float wv[4] = {wq.x, wq.y, wq.z, wq.w};
     uint32_t part = 0u;  // this lane's four nibbles in their place in the group's 32-bit word
-    uint16_t ep[3][4];   // the three bf16 parts of -E for this lane's four elements
+    float e4[4];         // E of this lane's four elements
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int j = 4 * q + t;
@@ -139,28 +122,9 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
       part |= ((neg << 3) | k) << (4 * (j & 7));
       float what = __fmul_rn(d.sg, __fmul_rn(e2m1_from_raw(k << 22), l));  // s_g (l q), l q exact
       if (neg) what = -what;
-      const float e = __fdiv_rn(__fsub_rn(wv[t], what), U[(col + j) * n + col + j]);
-      uint16_t pp[3];
-      split3(-e, pp);
-      ep[0][t] = pp[0];
-      ep[1][t] = pp[1];
-      ep[2][t] = pp[2];
+      e4[t] = __fdiv_rn(__fsub_rn(wv[t], what), U[(col + j) * n + col + j]);
     }
-    if (active) {
-      uint2 v[3];
-#pragma unroll
-      for (int p3 = 0; p3 < 3; ++p3)
-        v[p3] = make_uint2((uint32_t)ep[p3][0] | ((uint32_t)ep[p3][1] << 16),
-                           (uint32_t)ep[p3][2] | ((uint32_t)ep[p3][3] << 16));
-      uint2* row = reinterpret_cast<uint2*>(A + r * 6 * (int64_t)B + 16 * i + 4 * q);
-      const int seg = B / 4;  // one segment, in 8-byte words
-      row[0] = v[0];
-      row[seg] = v[0];
-      row[2 * seg] = v[1];
-      row[3 * seg] = v[0];
-      row[4 * seg] = v[1];
-      row[5 * seg] = v[2];
-    }
+    if (active) store_split3x4(A + r * 3 * (int64_t)B + 16 * i + 4 * q, B, e4);
     const uint32_t word = part | __shfl_xor_sync(0xFFFFFFFFu, part, 1);  // lanes 0-1: word 0, 2-3: word 1
     const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, word, 2);
     if (active && q == 0) {
@@ -170,8 +134,9 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
   }
 }
 
-// B' [nn, 6B] from U[col0 + k, c1 + j] (segments U1, U2, U1, U3, U2, U1), transposed through
-// 32 x 32 shared-memory tiles so that the reads of U and the writes of B' are coalesced
+// The update's other operand [nn, 3 B] (row j: the three bf16 parts of U[col0 .. col0 + B, c1 + j]),
+// transposed through 32 x 32 shared-memory tiles so that the reads of U and the writes are
+// coalesced
 __global__ void __launch_bounds__(256) split_u_kernel(const float* __restrict__ U, int64_t n, int64_t col0, int B,
                                                       int64_t c1, uint16_t* __restrict__ Bt) {
   __shared__ float t[32][33];
@@ -189,13 +154,10 @@ __global__ void __launch_bounds__(256) split_u_kernel(const float* __restrict__ 
     if (c1 + j < n && k < B) {
       uint16_t p[3];
       split3(t[tx][jj], p);
-      uint16_t* row = Bt + j * 6 * B + k;
+      uint16_t* row = Bt + j * 3 * B + k;
       row[0] = p[0];
       row[B] = p[1];
-      row[2 * B] = p[0];
-      row[3 * B] = p[2];
-      row[4 * B] = p[1];
-      row[5 * B] = p[0];
+      row[2 * B] = p[2];
     }
   }
 }
@@ -275,7 +237,7 @@ cudaError_t acquire_look_ahead(cudaStream_t stream, LookAheadLease* lease) {
 // A6 and B6 hold two buffers each: A' [m, 6 B] and B' [n, 6 B] bf16.
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
                                const float* global_scale, const uint8_t* dead, int block, int down, int up,
-                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* A6, uint16_t* B6,
+                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
                                cudaStream_t stream) {
   DeviceInfo info;
   cudaError_t err = current_device_info(&info);
@@ -286,8 +248,8 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   const int64_t groups = m * (B / 16);
   const unsigned qb = (unsigned)std::min<int64_t>((groups * 4 + 127) / 128, (int64_t)info.sm_count * 16);
-  uint16_t* Abuf[2] = {A6, A6 + m * 6 * B};
-  uint16_t* Bbuf[2] = {B6, B6 + n * 6 * B};
+  uint16_t* Abuf[2] = {Es, Es + m * 3 * B};
+  uint16_t* Bbuf[2] = {Us, Us + n * 3 * B};
   auto quantize = [&](int64_t b, cudaStream_t s) {
     block_kernel<<<qb, 128, 0, s>>>(Wf, m, n, b * B, block, h, U, global_scale, down, up, codes,
                                     reinterpret_cast<uint2*>(packed), Abuf[b & 1]);
@@ -310,7 +272,7 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
       if (b + 1 == nb) break;
       const int64_t c1 = (b + 1) * B, nn = n - c1;
       if ((err = split_u(b, stream)) != cudaSuccess) return err;
-      if ((err = launch_gemm_accumulate(Abuf[b & 1], Bbuf[b & 1], m, nn, 6 * B, Wf + c1, n, stream)) != cudaSuccess)
+      if ((err = launch_split_update(Abuf[b & 1], Bbuf[b & 1], m, nn, B, Wf + c1, n, stream)) != cudaSuccess)
         return err;
     }
     return cudaSuccess;
@@ -335,14 +297,14 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
     if ((err = cudaEventRecord(ev_q[x], stream)) != cudaSuccess) return err;
     if ((err = cudaStreamWaitEvent(stream, ev_su[x], 0)) != cudaSuccess) return err;
     if (b >= 1 && (err = cudaStreamWaitEvent(stream, ev_gb[x ^ 1], 0)) != cudaSuccess) return err;
-    if ((err = launch_gemm_accumulate(Abuf[x], Bbuf[x], m, std::min<int64_t>(B, nn), 6 * B, Wf + c1, n, stream)) !=
+    if ((err = launch_split_update(Abuf[x], Bbuf[x], m, std::min<int64_t>(B, nn), B, Wf + c1, n, stream)) !=
         cudaSuccess)
       return err;
     if ((err = cudaEventRecord(ev_ga[x], stream)) != cudaSuccess) return err;
     // ---- the second stream
     if ((err = cudaStreamWaitEvent(side, ev_q[x], 0)) != cudaSuccess) return err;
-    if (nn > B && (err = launch_gemm_accumulate(Abuf[x], Bbuf[x] + B * 6 * B, m, nn - B, 6 * B, Wf + c1 + B, n,
-                                                side)) != cudaSuccess)
+    if (nn > B && (err = launch_split_update(Abuf[x], Bbuf[x] + B * 3 * B, m, nn - B, B, Wf + c1 + B, n,
+                                             side)) != cudaSuccess)
       return err;
     if ((err = cudaEventRecord(ev_gb[x], side)) != cudaSuccess) return err;
     if (b + 2 < nb) {  // U's split for the next block, once both updates of block b - 1 have read its buffer

@@ -105,22 +105,29 @@ int64_t gptq_factor_padded(int64_t n);
 size_t gptq_factor_workspace(int64_t n);
 cudaError_t launch_gptq_factor(const float* H, int64_t n, int64_t ld_h, float damp, float* U, uint8_t* dead,
                                int32_t* info, void* workspace, cudaStream_t stream);
-// C[m, nn] (row stride ld_c, fp32) += A B^T on the tensor cores, with A [m, k] and B [nn, k]
-// bf16, rows of k elements contiguous (k % 8 == 0, 16-byte aligned bases); every tile.
-// programmatic: launched with programmatic dependent launch (the kernel waits for the
-// previous kernel on the stream before its first load, and lets the next one be scheduled).
-cudaError_t launch_gemm_accumulate(const void* a, const void* b, int64_t m, int64_t nn, int64_t k, float* C,
-                                   int64_t ld_c, cudaStream_t stream, bool programmatic = false);
+// C [rows, cols] (row stride ld, fp32) -= A B^T on the tensor cores with fp32-level accuracy; A
+// [rows, K] and B [cols, K] as three bf16 parts per row (split3.cuh), segments of K, K % 8 == 0,
+// 16-byte aligned bases.
+cudaError_t launch_split_update(const void* a, const void* b, int64_t rows, int64_t cols, int64_t K, float* C,
+                                int64_t ld, cudaStream_t stream);
+// One step of the factor's sweep (K = 128): operand = [L_:j ; X_j,:^T] (rows + xcols rows of three
+// parts); the trailing square C [rows, rows] (its lower triangle) and the inverse X [rows, xcols]
+// (rows below the diagonal block) both -= L_:j [.]^T, and the next diagonal block (C's first) is
+// factored and its inverse written at X's columns order0 .. order0 + 127.  Launched with
+// programmatic dependent launch.
+cudaError_t launch_factor_update(const void* operand, int64_t rows, int64_t xcols, float* C, float* X, int64_t ld,
+                                 int32_t order0, int32_t* info, cudaStream_t stream);
 
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
                                const float* global_scale, const uint8_t* dead, int block, int down, int up,
-                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* A6, uint16_t* B6,
+                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
                                cudaStream_t stream);
 
 // Sticky device error flags of each translation unit (bit 0: a bounded wait ran out);
 // cleared on read.
 cudaError_t read_hessian_device_error(uint32_t* flags);
 cudaError_t read_output_error_device_error(uint32_t* flags);
+cudaError_t read_update_device_error(uint32_t* flags);
 cudaError_t read_selftest_device_error(uint32_t* flags);
 
 // One CTA waits at most `polls` polls on an mbarrier that nothing arrives on.

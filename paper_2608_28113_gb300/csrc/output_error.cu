@@ -44,7 +44,6 @@ constexpr int kGemmThreads = 320;  // TMA warp, MMA warp, 8 epilogue warps
 constexpr uint32_t kTileABytes = kBM * kBK * 2;  // 16 KB
 constexpr uint32_t kTileBBytes = kBN * kBK * 2;  // 32 KB
 constexpr uint32_t kStageBytes = kTileABytes + kTileBBytes;
-constexpr uint32_t kTmemCols = kBN;  // fp32 accumulator: 128 lanes x 256 columns
 // Full Hessian (modes 1, 3) and output error (mode 0): the tensor cores accumulate in fp32
 // with an error that grows with the accumulation length (the Hessian's diagonal comes out
 // low by about 0.9 u per K = 16 step, measured), so each tile's K loop is cut into
@@ -57,37 +56,11 @@ constexpr uint32_t kTmemCols = kBN;  // fp32 accumulator: 128 lanes x 256 column
 constexpr int kSegBlocks = 32;
 constexpr uint32_t kTmemColsSeg = 2 * kBN;
 constexpr uint32_t kGemmSmemBytes = kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers */;
-// the GPTQ update also stages its epilogue: barriers in a 1 KB block (keeping the staging
-// buffers 1 KB aligned for the 128-byte swizzle), then 4 KB per epilogue warp
-constexpr uint32_t kUpdateSmemBytes = kStages * kStageBytes + 1024 /* alignment */ + 1024 + 8 * 4096;
 constexpr uint32_t kIdesc = idesc_bf16_f32(kBM, kBN);
 constexpr uint32_t kIdescMN = idesc_bf16_f32_mn(kBM, kBN);
 constexpr uint32_t kBoxBytes = 64 * kBK * 2;  // mode 3: one 64-channel x 64-token TMA box
 
 __device__ uint32_t g_output_error_flags = 0;
-
-// ---------------------------------------------------------------- TMA reduce-add
-// The GPTQ update's epilogue adds each tile into the running weights with TMA: a warp
-// stages 32 rows x 32 fp32 columns (4 KB, 128-byte swizzled, as the tensor map says) and
-// one lane issues a bulk reduce-add, which the L2 applies in fp32 round-to-nearest without
-// the SM reading the weights.  The coordinates are (column, row), column a multiple of 4.
-constexpr uint32_t kStageRows = 32, kStageCols = 32;
-constexpr uint32_t kStageBufBytes = kStageRows * kStageCols * 4;  // per epilogue warp
-
-__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, const void* src, int32_t c0, int32_t c1) {
-  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(c0), "r"(c1), "r"(smem_addr(src))
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// every committed bulk operation has finished reading shared memory
-__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// every committed bulk operation has completed
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 
 // ---------------------------------------------------------------- residual
 __device__ __forceinline__ uint32_t bf16x2_pack(__nv_bfloat16 lo, __nv_bfloat16 hi) {
@@ -163,8 +136,7 @@ __device__ __forceinline__ float sum_squares32(const uint32_t (&r)[32]) {
 
 // kMode 0: the sum-of-squares GEMM of the output error (K runs over [X | X], kb_half
 // blocks per half).  kMode 1: H[rows, cols] += A B^T over kb_half K blocks, both operands
-// rows of X^T, tiles wholly below the diagonal skipped.  kMode 2: C[rows, cols] += A B^T
-// over kb_half K blocks, every tile (the GPTQ update).  kMode 3: kMode 1 read from X itself
+// rows of X^T, tiles wholly below the diagonal skipped.  kMode 3: kMode 1 read from X itself
 // ([tokens, n], channels contiguous): each stage loads 64-channel x 64-token boxes and
 // the MMAs take both operands MN-major, so no transpose is needed.
 // Tile t of a persistent GEMM's sequence (tiles_n column tiles per row of tiles) in groups of
@@ -184,7 +156,7 @@ __device__ __forceinline__ void raster_tile(int t, int tiles_n, int tiles_total,
 template <int kMode>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
-            const __grid_constant__ CUtensorMap cmap, int kb_half, int tiles_n, int tiles_total,
+            int kb_half, int tiles_n, int tiles_total,
             double* __restrict__ partials, float* __restrict__ H, int64_t h_rows, int64_t h_cols, int64_t ld_h) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -192,28 +164,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   uint8_t* tile_b = smem + kStages * kTileABytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
   uint64_t* empty = full + kStages;
-  uint64_t* acc_ready = empty + kStages;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_ready + 1);
+  uint64_t* seg_full = empty + kStages;  // a segment's partial is complete
+  uint64_t* seg_empty = seg_full + 1;    // the partial has been read out
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(seg_empty + 1);
   uint32_t* failed = tmem_slot + 1;
-  uint64_t* seg_full = acc_ready + 2;  // segmented modes: a segment's partial is complete
-  uint64_t* seg_empty = seg_full + 1;  // segmented modes: the partial has been read out
-  uint64_t* tacc_full = seg_empty + 1;  // mode 2: accumulator a holds a finished tile
-  uint64_t* tacc_empty = tacc_full + 2;  // mode 2: accumulator a has been read out
   double* warp_sum = reinterpret_cast<double*>(smem + kStages * kStageBytes + 128);
   constexpr bool kHessian = kMode == 1 || kMode == 3;
-  // K loops cut into accumulation segments folded in TMEM: the Hessian (K = tokens) and the
-  // output error (K = 2 n); the GPTQ update's K = 6 B is a single segment anyway
-  constexpr bool kSegmented = kMode != 2;
-  // The GPTQ update and the output error are persistent: a CTA takes tiles blockIdx.x,
-  // + gridDim.x, ...  The update alternates two 256-column accumulators, so a tile's
-  // epilogue (the TMA reduce-add into the running weights) runs alongside the next tile's
-  // loads and MMAs.  The output error's segments run on across its tiles (one segment
-  // counter), so the MMAs of a tile's first segment start as soon as the previous tile's
-  // last partial has been read out, alongside that tile's sum of squares.  The Hessian modes
-  // take one tile per CTA.
-  constexpr bool kPersistent = kMode == 2 || kMode == 0;
-  constexpr bool kTwoAcc = kMode == 2;
-  constexpr uint32_t kCols = (kSegmented || kPersistent) ? kTmemColsSeg : kTmemCols;
+  // The output error is persistent: a CTA takes tiles blockIdx.x, + gridDim.x, ...  Its segments
+  // run on across its tiles (one segment counter), so the MMAs of a tile's first segment start
+  // as soon as the previous tile's last partial has been read out, alongside that tile's sum of
+  // squares.  The Hessian modes take one tile per CTA.
+  constexpr bool kPersistent = kMode == 0;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = kPersistent ? (tiles_total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 1;
@@ -229,34 +190,21 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(acc_ready, 1);
     mbar_init(seg_full, 1);
     mbar_init(seg_empty, 256);  // every epilogue thread arrives
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(&tacc_full[a], 1);
-      mbar_init(&tacc_empty[a], 256);
-    }
     *failed = 0u;
     mbar_fence_init();
     prefetch_tensormap(&xmap);
     prefetch_tensormap(&wmap);
   }
   if (warp == 1) {
-    tmem_alloc(smem_addr(tmem_slot), kCols);
+    tmem_alloc(smem_addr(tmem_slot), kTmemColsSeg);
     tmem_relinquish();
   }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_d = *tmem_slot;
-  if (kMode == 2) {
-    // launched with programmatic dependent launch by the factor's sweep: let the next kernel
-    // be scheduled (after the TMEM allocation), then wait for the previous one's writes
-    // before the first load; without the launch attribute both are no-ops
-    pdl_launch_dependents();
-    pdl_wait_primary();
-  }
-
   if (warp == 0) {
     if (lane == 0) {
       uint64_t policy;
@@ -296,30 +244,22 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      // the segmented modes: segments of kSegBlocks K blocks, each accumulated from zero;
-      // the GPTQ update: one segment over its short K loop, per tile
-      const int seg_blocks = kSegmented ? kSegBlocks : (kb_total > 0 ? kb_total : 1);
-      const int nseg = (kb_total + seg_blocks - 1) / seg_blocks;
+      // segments of kSegBlocks K blocks, each accumulated from zero
+      const int nseg = (kb_total + kSegBlocks - 1) / kSegBlocks;
       bool ok = true;
       for (int i = 0; i < ntiles && ok; ++i) {
-        const uint32_t acc = kTwoAcc ? (uint32_t)(i & 1) : 0u;
-        // the accumulator's previous tile (two back) must have been read out of TMEM
-        if (kTwoAcc && i >= 2 && !mbar_wait(&tacc_empty[acc], (uint32_t)((i >> 1) - 1) & 1u)) {
-          atomicOr(failed, 1u);
-          break;
-        }
         for (int seg = 0; seg < nseg && ok; ++seg) {
           // the previous segment's partial (of this tile or the one before) must have been
           // read out of TMEM
           const int gs = i * nseg + seg;
-          if (kSegmented && gs >= 1 && !mbar_wait(seg_empty, (uint32_t)(gs - 1) & 1u)) {
+          if (gs >= 1 && !mbar_wait(seg_empty, (uint32_t)(gs - 1) & 1u)) {
             atomicOr(failed, 1u);
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          const uint32_t d = tmem_d + acc * kBN;
-          const int kb0 = seg * seg_blocks, kb1 = min(kb_total, kb0 + seg_blocks);
+          const uint32_t d = tmem_d;
+          const int kb0 = seg * kSegBlocks, kb1 = min(kb_total, kb0 + kSegBlocks);
           for (int kb = kb0; kb < kb1; ++kb) {
             const int g = i * kb_total + kb;
             const int s = g % kStages;
@@ -347,7 +287,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
             umma_commit(smem_addr(&empty[s]));
           }
           // fires once every MMA issued above has completed
-          if (ok) umma_commit(smem_addr(kSegmented ? seg_full : (kTwoAcc ? &tacc_full[acc] : acc_ready)));
+          if (ok) umma_commit(smem_addr(seg_full));
         }
       }
     }
@@ -359,7 +299,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     const uint32_t quarter = (uint32_t)(warp & 3);
     const uint32_t cbase = (uint32_t)((warp - 2) >> 2) * kHalf;
     const uint32_t lane_base = (quarter * 32u) << 16;
-    const int nseg = kSegmented ? (kb_total + kSegBlocks - 1) / kSegBlocks : 1;
+    const int nseg = (kb_total + kSegBlocks - 1) / kSegBlocks;
     double acc = 0.0;
     bool alive = true;
     for (int i = 0; i < ntiles && alive; ++i) {
@@ -367,12 +307,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       const int tm = t / tiles_n, tn = t - tm * tiles_n;
       const int64_t row = (int64_t)tm * kBM + quarter * 32 + lane;
       const int64_t col0 = (int64_t)tn * kBN + cbase;
-      const uint32_t tacc = kTwoAcc ? (uint32_t)(i & 1) : 0u;
       for (int seg = 0; seg < nseg; ++seg) {
-        uint64_t* ready = kSegmented ? seg_full : (kTwoAcc ? &tacc_full[tacc] : acc_ready);
-        const uint32_t parity =
-            kSegmented ? (uint32_t)(i * nseg + seg) & 1u : (kTwoAcc ? (uint32_t)(i >> 1) & 1u : 0u);
-        if (!mbar_wait(ready, parity)) {
+        if (!mbar_wait(seg_full, (uint32_t)(i * nseg + seg) & 1u)) {
           atomicOr(failed, 1u);
           alive = false;
           break;
@@ -382,16 +318,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         uint32_t p[kHalf];
 #pragma unroll
         for (int c = 0; c < kHalf; c += 32)
-          tmem_ld_32x32b_x32(tmem_d + tacc * kBN + lane_base + cbase + (uint32_t)c,
+          tmem_ld_32x32b_x32(tmem_d + lane_base + cbase + (uint32_t)c,
                              *reinterpret_cast<uint32_t(*)[32]>(p + c));
         tmem_ld_wait();
-        if ((kSegmented && (!last || kPersistent)) || kTwoAcc) {
+        if (!last || kPersistent) {
           // the partial is in registers: the MMAs may go on with the next segment (of this
-          // tile or the next), or the tile after next may use this accumulator
+          // tile or the next)
           tc_fence_before_sync();
-          mbar_arrive(kTwoAcc ? &tacc_empty[tacc] : seg_empty);
+          mbar_arrive(seg_empty);
         }
-        if (kSegmented && seg > 0) {
+        if (seg > 0) {
           // fold into the running sum (TMEM columns [256, 512)), fp32 round-to-nearest
 #pragma unroll
           for (int c = 0; c < kHalf; c += 32) {
@@ -403,7 +339,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
               p[c + j] = __float_as_uint(__fadd_rn(__uint_as_float(q[j]), __uint_as_float(p[c + j])));
           }
         }
-        if (kSegmented && !last) {
+        if (!last) {
 #pragma unroll
           for (int c = 0; c < kHalf; c += 32)
             tmem_st_32x32b_x32(tmem_d + lane_base + kBN + cbase + (uint32_t)c, *reinterpret_cast<uint32_t(*)[32]>(p + c));
@@ -414,31 +350,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
           // the output error: the sum of squares of the complete tile
 #pragma unroll
           for (int c = 0; c < kHalf; c += 32) acc += (double)sum_squares32(*reinterpret_cast<uint32_t(*)[32]>(p + c));
-          continue;
-        }
-        if (kTwoAcc) {
-          // the GPTQ update: staged 32 x 32 boxes reduce-added into C by TMA.  Row `lane`
-          // of a box holds 128 bytes; the 128-byte swizzle puts its 16-byte chunk k at
-          // k ^ (lane & 7), so a warp's stores hit every bank once.
-          uint8_t* stage = smem + kStages * kStageBytes + 1024 + (uint32_t)(warp - 2) * kStageBufBytes;
-          const int64_t row0 = (int64_t)tm * kBM + quarter * 32;
-#pragma unroll
-          for (int c = 0; c < kHalf; c += 32) {
-            // the previous box must have been read out of the buffer
-            if (lane == 0) bulk_wait_read();
-            __syncwarp();
-            float4* rowp = reinterpret_cast<float4*>(stage + lane * 128);
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              rowp[k ^ (lane & 7)] = make_float4(__uint_as_float(p[c + 4 * k]), __uint_as_float(p[c + 4 * k + 1]),
-                                                 __uint_as_float(p[c + 4 * k + 2]), __uint_as_float(p[c + 4 * k + 3]));
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0 && row0 < h_rows && col0 + c < h_cols) {
-              tma_reduce_add_2d(&cmap, stage, (int32_t)(col0 + c), (int32_t)row0);
-              bulk_commit();
-            }
-          }
           continue;
         }
         // the Hessian: the tile row added into H
@@ -462,8 +373,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         }
       }
     }
-    // the update's reduce-adds complete before the CTA ends
-    if (kTwoAcc && lane == 0) bulk_wait_all();
     if (!kAccum) {
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
@@ -497,7 +406,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   }
   if (warp == 1) {
     tc_fence_after_sync();
-    tmem_dealloc(tmem_d, kCols);
+    tmem_dealloc(tmem_d, kTmemColsSeg);
   }
 }
 
@@ -595,7 +504,7 @@ cudaError_t launch_output_error(const void* x, int64_t tokens, int64_t n, int64_
   if ((err = current_device_info(&info)) != cudaSuccess) return err;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(tiles, info.sm_count));
   gemm_kernel<0><<<(unsigned)grid, kGemmThreads, kGemmSmemBytes, stream>>>(
-      xmap, wmap, wmap, (int)(n_pad / kBK), (int)tiles_n, (int)tiles, partials, nullptr, 0, 0, 0);
+      xmap, wmap, (int)(n_pad / kBK), (int)tiles_n, (int)tiles, partials, nullptr, 0, 0, 0);
   err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   reduce_kernel<<<1, 256, 0, stream>>>(partials, grid, out);
@@ -625,7 +534,7 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
     err = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<3>), (int)kGemmSmemBytes);
     if (err != cudaSuccess) return err;
     gemm_kernel<3><<<(unsigned)tiles, kGemmThreads, kGemmSmemBytes, stream>>>(
-        map, map, map, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
+        map, map, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
     return cudaGetLastError();
   }
   // X with rows that are not 16-byte aligned: transposed first (tokens contiguous per
@@ -651,59 +560,7 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
       ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<1>), (int)kGemmSmemBytes);
   if (attr_status != cudaSuccess) return attr_status;
   gemm_kernel<1><<<(unsigned)tiles, kGemmThreads, kGemmSmemBytes, stream>>>(
-      amap, bmap, bmap, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_gemm_accumulate(const void* a, const void* b, int64_t m, int64_t nn, int64_t k, float* C,
-                                   int64_t ld_c, cudaStream_t stream, bool programmatic) {
-  EncodeTiledFn encode = nullptr;
-  cudaError_t err = encode_tiled_fn(&encode);
-  if (err != cudaSuccess) return err;
-  CUtensorMap amap, bmap, cmap;
-  const cuuint64_t adims[2] = {(cuuint64_t)k, (cuuint64_t)m};
-  const cuuint64_t bdims[2] = {(cuuint64_t)k, (cuuint64_t)nn};
-  const cuuint64_t strides[1] = {(cuuint64_t)k * 2};
-  const cuuint32_t estr[2] = {1, 1};
-  const cuuint32_t abox[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
-  const cuuint32_t bbox[2] = {(cuuint32_t)kBK, (cuuint32_t)kBN};
-  if (encode(&amap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a), adims, strides, abox, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-      encode(&bmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(b), bdims, strides, bbox, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  // C [m, nn] fp32 (row stride ld_c), reduce-added in 32 x 32 boxes
-  const cuuint64_t cdims[2] = {(cuuint64_t)nn, (cuuint64_t)m};
-  const cuuint64_t cstrides[1] = {(cuuint64_t)ld_c * 4};
-  const cuuint32_t cbox[2] = {kStageCols, kStageRows};
-  if ((reinterpret_cast<uintptr_t>(C) & 15) != 0 || (ld_c * 4) % 16 != 0) return cudaErrorInvalidValue;
-  if (encode(&cmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, C, cdims, cstrides, cbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
-      CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  err = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<2>), (int)kUpdateSmemBytes);
-  if (err != cudaSuccess) return err;
-  const int64_t tiles_n = (nn + kBN - 1) / kBN;
-  const int64_t tiles = ((m + kBM - 1) / kBM) * tiles_n;
-  // persistent: one CTA per SM (the shared-memory ring allows no more), tiles strided
-  DeviceInfo info;
-  if ((err = current_device_info(&info)) != cudaSuccess) return err;
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(tiles, info.sm_count));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(kGemmThreads, 1, 1);
-  cfg.dynamicSmemBytes = kUpdateSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = programmatic ? 1 : 0;
-  err = cudaLaunchKernelEx(&cfg, gemm_kernel<2>, amap, bmap, cmap, (int)((k + kBK - 1) / kBK), (int)tiles_n,
-                           (int)tiles, (double*)nullptr, C, m, nn, ld_c);
-  if (err != cudaSuccess) return err;
+      amap, bmap, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
   return cudaGetLastError();
 }
 

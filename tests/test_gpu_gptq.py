@@ -141,6 +141,22 @@ def test_factor_sizes_across_block_boundaries(n, tokens):
     assert hs.hscale_device_error_flags() == 0
 
 
+@pytest.mark.parametrize("power", [-104, 90])
+def test_factor_of_a_scaled_matrix(power):
+    """U of 2^power H is 2^(-power/2) U.  At these powers the pivots leave the range of the quick
+    reciprocals of the diagonal blocks (2^-100 to 2^100), so their full-range form runs; both
+    forms are within about 2^-22, and the factor's error grows with the condition of the damped H,
+    so the bound is that of the oracle comparison above."""
+    n = 300
+    x = calib(n, 900, 17)
+    H32 = oracle_H(x, n).astype(np.float32)
+    U, dead, info = gpu_factor(H32)
+    Us, deads, infos = gpu_factor(np.ldexp(H32, power).astype(np.float32))
+    assert np.all(info == 0) and np.all(infos == 0) and np.array_equal(dead, deads)
+    d = np.ldexp(Us, power // 2) - U
+    assert np.linalg.norm(d) <= 1e-4 * np.linalg.norm(U)
+
+
 def test_factor_reports_a_matrix_that_is_not_positive_definite():
     """A symmetric matrix with a negative eigenvalue that the damping does not lift: info[0]
     names a failed pivot (1-based, in the reversed order); U is then unspecified."""
