@@ -39,8 +39,7 @@
  * Conventions shared by every entry point
  * ---------------------------------------
  * - All pointers except `stream` are DEVICE pointers owned by the caller; the
- *   library allocates and frees no memory (hscale_gptq_hscale keeps one stream and a
- *   few events per device context, see there).  Work is enqueued on `stream` (a
+ *   library allocates and frees no memory.  Work is enqueued on `stream` (a
  *   cudaStream_t passed as void*, NULL = legacy default stream) and nothing
  *   synchronises: results are ready when the stream reaches them.
  * - Matrices are row-major.  W is [m, n] bfloat16 with contiguous rows; groups of 16
@@ -461,15 +460,11 @@ int hscale_output_error(const void* x_bf16, int64_t tokens, int64_t n, int64_t l
  *    accuracy (on the tensor cores: three-way bf16 splits of E and U, the six products
  *    above 2^-24 relative, fp32 accumulation).  Writes codes_out [m, n/16] and packed_out
  *    [m, n/2] (8-byte aligned) as hscale_refine_scales does.  The workspace
- *    (hscale_gptq_workspace_bytes) holds the running weights and two buffers of each
- *    split operand.  With more than one block the call works ahead: the update of the
- *    next block's columns runs on `stream` and the rest of each update on a second stream
- *    of the library, alongside the next block's quantization; events order the two, every
- *    weight receives its updates in block order (the same bits on every run), and the
- *    call's work on `stream` ends after all of it.  The library creates that stream and
- *    its events on the first such call in each device context and keeps them; a first
- *    call made while `stream` is being captured (which may not create them) runs every
- *    block on `stream` instead, with the same results.  Calls are enqueued one at a time.
+ *    (hscale_gptq_workspace_bytes) holds the running weights and the split operands.
+ *    Blocks are taken in panels of up to 512 columns (a wider block is a panel of its own):
+ *    inside a panel each block's update reaches the panel's columns at once, and the columns
+ *    right of it take the panel's update at its end, in the same order for every weight on
+ *    every run (the same bits).  Everything runs on `stream`.
  */
 size_t hscale_hessian_full_workspace_bytes(int64_t tokens, int64_t n);
 int hscale_hessian_full_accumulate(const void* x_bf16, int64_t tokens, int64_t n, int64_t ld_x, float* H,

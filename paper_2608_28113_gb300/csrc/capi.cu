@@ -4,6 +4,7 @@
 // then calls the launchers in hessian.cu / scales.cu.  No exception crosses the ABI.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -73,12 +74,13 @@ int hscale_abi_version(void) { return 4; }
 
 int hscale_device_error_flags(uint32_t* flags) {
   if (flags == nullptr) return HSCALE_ERR_NULL;
-  uint32_t a = 0, b = 0, c = 0, d = 0;
+  uint32_t a = 0, b = 0, c = 0, d = 0, e = 0;
   cudaError_t err = hscale::read_hessian_device_error(&a);
   if (err == cudaSuccess) err = hscale::read_output_error_device_error(&b);
   if (err == cudaSuccess) err = hscale::read_selftest_device_error(&c);
   if (err == cudaSuccess) err = hscale::read_update_device_error(&d);
-  *flags = a | b | c | d;
+  if (err == cudaSuccess) err = hscale::read_gptq_device_error(&e);
+  *flags = a | b | c | d | e;
   return from_cuda(err);
 }
 
@@ -326,12 +328,19 @@ namespace {
 inline int64_t round256(int64_t bytes) { return (bytes + 255) / 256 * 256; }
 }  // namespace
 
-// running weights (fp32 m x n) and two buffers each of the bf16 split operands of the
-// update: E (m x 3 block, in regions of m x 6 block) and U's rows (n x 3 block, likewise)
+// running weights (fp32 m x n) and the bf16 split operands of the update: the errors
+// (m rows of three parts) and U's rows (n rows), each part as wide as the update's K; never less
+// than two buffers of 6 block per row
+namespace {
+inline int64_t gptq_operand_row(int64_t n, int64_t block) {
+  return std::max<int64_t>(3 * hscale::gptq_update_cols(n, block), 12 * block);
+}
+}  // namespace
+
 size_t hscale_gptq_workspace_bytes(int64_t m, int64_t n, int32_t block) {
   if (m <= 0 || n <= 0 || block <= 0) return 0;
-  const int64_t b = block;
-  return (size_t)(round256(m * n * 4) + round256(2 * m * 6 * b * 2) + round256(2 * n * 6 * b * 2));
+  const int64_t row = gptq_operand_row(n, block);
+  return (size_t)(round256(m * n * 4) + round256(m * row * 2) + round256(n * row * 2));
 }
 
 int hscale_gptq_hscale(const void* w_bf16, int64_t m, int64_t n, const float* U, const float* h,
@@ -350,10 +359,10 @@ int hscale_gptq_hscale(const void* w_bf16, int64_t m, int64_t n, const float* U,
   if (workspace == nullptr || workspace_bytes < hscale_gptq_workspace_bytes(m, n, block) || !aligned(workspace, 256))
     return HSCALE_ERR_WORKSPACE;
   uint8_t* base = static_cast<uint8_t*>(workspace);
-  const int64_t b = block;
+  const int64_t row = gptq_operand_row(n, block);
   float* Wf = reinterpret_cast<float*>(base);
   uint16_t* Es = reinterpret_cast<uint16_t*>(base + round256(m * n * 4));
-  uint16_t* Us = reinterpret_cast<uint16_t*>(base + round256(m * n * 4) + round256(2 * m * 6 * b * 2));
+  uint16_t* Us = reinterpret_cast<uint16_t*>(base + round256(m * n * 4) + round256(m * row * 2));
   return from_cuda(hscale::launch_gptq_hscale(w_bf16, m, n, U, h, global_scale, dead, block, down, up, codes_out,
                                               packed_out, Wf, Es, Us, as_stream(stream)));
 }

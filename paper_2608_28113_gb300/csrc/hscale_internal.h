@@ -5,8 +5,6 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 namespace hscale {
 
 struct DeviceInfo {
@@ -62,19 +60,6 @@ cudaError_t encode_tiled_fn(EncodeTiledFn* out);
 // created again after cudaDeviceReset gets a new id.
 cudaError_t current_context_id(unsigned long long* id);
 
-// The library's second stream and its events in the current device context, for calls that
-// work ahead on it (created on first use and kept).  The lease holds the library's mutex:
-// release it (destroy the lease) only after the call has enqueued all its work.  side is
-// null when they do not exist yet and `stream` is being captured (they may not be created
-// then): the call then runs on `stream` alone.
-constexpr int kLookAheadEvents = 10;
-struct LookAheadLease {
-  std::unique_lock<std::mutex> lock;
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev[kLookAheadEvents] = {};
-};
-cudaError_t acquire_look_ahead(cudaStream_t stream, LookAheadLease* lease);
-
 // cudaFuncAttributeMaxDynamicSharedMemorySize = bytes and the maximum shared-memory
 // carveout for kernel `func` on the current device, set once per (kernel, device) and
 // remembered, so that every GPU of a process gets it (a function attribute belongs to one
@@ -118,6 +103,8 @@ cudaError_t launch_split_update(const void* a, const void* b, int64_t rows, int6
 cudaError_t launch_factor_update(const void* operand, int64_t rows, int64_t xcols, float* C, float* X, int64_t ld,
                                  int32_t order0, int32_t* info, cudaStream_t stream);
 
+// Algorithm 3's block loop.  Wf: m x n floats; Es and Us: m and n rows of 3 gptq_update_cols() bf16.
+int64_t gptq_update_cols(int64_t n, int64_t block);
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
                                const float* global_scale, const uint8_t* dead, int block, int down, int up,
                                uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
@@ -128,6 +115,7 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
 cudaError_t read_hessian_device_error(uint32_t* flags);
 cudaError_t read_output_error_device_error(uint32_t* flags);
 cudaError_t read_update_device_error(uint32_t* flags);
+cudaError_t read_gptq_device_error(uint32_t* flags);
 cudaError_t read_selftest_device_error(uint32_t* flags);
 
 // One CTA waits at most `polls` polls on an mbarrier that nothing arrives on.

@@ -233,6 +233,45 @@ def test_gptq_one_block_and_diagonal_factor_reduce_to_the_search():
     exact_outside_near_ties(codes, packed, ref, "diagonal factor")
 
 
+@pytest.mark.parametrize("m,n,block", [
+    (1, 64, 16),        # one row; four blocks in one panel
+    (33, 1104, 48),     # panels of 480 columns and a ragged last one; rows of three CTAs, the last ragged
+    (17, 528, 16),      # a last panel of a single block
+    (40, 768, 256),     # the widest block with an update inside the panel
+    (24, 1024, 512),    # a block per panel
+    (20, 1152, 576),    # a block wider than a panel
+    (2448, 256, 64),    # more than 16 rows per SM: 32 rows a CTA
+])
+def test_gptq_panel_shapes(m, n, block):
+    """Panel, block and row counts where the block loop's kernels change shape, against the
+    oracle, under the rules above."""
+    w, x, H, U32, h32, dead = layer_inputs(m, n, 500 + block, tokens=2 * n)
+    wb = bits(w)
+    s_g, _ = oracle.global_scale(wb)
+    codes, packed = gpu_gptq(w, U32, h32, s_g, block, 4, 4, dead=dead)
+    ref = oracle.gptq_hscale(wb, U32.astype(np.float64), h32, s_g, block, 4, 4, dead=dead)
+    nb = block // 16
+    first = {k: ref[k][:, :nb] for k in ("codes", "near_tie")}
+    first["packed"] = ref["packed"][:, :block // 2]
+    exact_outside_near_ties(codes[:, :nb], packed[:, :block // 2], first, "first block")
+    assert float(np.mean(codes == ref["codes"])) >= 0.98
+    assert hs.hscale_device_error_flags() == 0
+
+
+def test_gptq_zero_groups_keep_the_initial_code():
+    """Groups that are all zero (dead channels) score zero under every code: the tie rule keeps
+    the initial code, 1, and the nibbles are zero."""
+    m, n, block = 40, 256, 64
+    w, x, H, U32, h32, dead = layer_inputs(m, n, 77)
+    dead = np.zeros(n, dtype=bool)
+    dead[96:128] = True
+    wb = bits(w)
+    s_g, _ = oracle.global_scale(wb)
+    Ud = np.diag(np.diag(U32)).astype(np.float32)  # nothing is propagated into the dead channels
+    codes, packed = gpu_gptq(w, Ud, h32, s_g, block, 4, 4, dead=dead)
+    assert np.all(codes[:, 6:8] == 1) and np.all(packed[:, 48:64] == 0)
+
+
 def test_full_size_gptq_q_proj_slice():
     """A 1024 x 4096 slice of the q_proj layer at full width with the full pipeline on the
     GPU (H on the tensor cores, the factor, block loop of 128 columns, k = 4) against
