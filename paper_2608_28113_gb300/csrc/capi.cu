@@ -133,7 +133,7 @@ int hscale_amax_bits(const void* w_bf16, int64_t m, int64_t n, uint32_t* amax_bi
 int hscale_global_scale_from_amax(const uint32_t* amax_bits, float* global_scale, void* stream) {
   if (amax_bits == nullptr || global_scale == nullptr) return HSCALE_ERR_NULL;
   if (!aligned(amax_bits, 4) || !aligned(global_scale, 4)) return HSCALE_ERR_ALIGN;
-  return from_cuda(hscale::launch_rtn_codes(nullptr, 0, 16, amax_bits, global_scale, nullptr, as_stream(stream)));
+  return from_cuda(hscale::launch_scale_from_amax(amax_bits, global_scale, as_stream(stream)));
 }
 
 size_t hscale_rtn_workspace_bytes(void) { return 256; }
@@ -147,13 +147,7 @@ int hscale_rtn_scales(const void* w_bf16, int64_t m, int64_t n, float* global_sc
   if (!aligned(global_scale, 4)) return HSCALE_ERR_ALIGN;
   if (workspace == nullptr || workspace_bytes < hscale_rtn_workspace_bytes()) return HSCALE_ERR_WORKSPACE;
   if (!aligned(workspace, 4)) return HSCALE_ERR_ALIGN;
-  cudaStream_t s = as_stream(stream);
-  uint32_t* amax = static_cast<uint32_t*>(workspace);
-  cudaError_t err = cudaMemsetAsync(amax, 0, sizeof(uint32_t), s);
-  if (err != cudaSuccess) return HSCALE_ERR_CUDA;
-  err = hscale::launch_amax(w_bf16, m * n, amax, s);
-  if (err != cudaSuccess) return HSCALE_ERR_CUDA;
-  return from_cuda(hscale::launch_rtn_codes(w_bf16, m, n, amax, global_scale, codes, s));
+  return from_cuda(hscale::launch_rtn_scales(w_bf16, m, n, workspace, global_scale, codes, as_stream(stream)));
 }
 
 int hscale_refine_scales(const void* w_bf16, const float* h, int64_t m, int64_t n,

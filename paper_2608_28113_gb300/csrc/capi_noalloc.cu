@@ -4,8 +4,8 @@
 // Some callers of this library cannot allocate device memory: a plugin or callback that
 // is handed only its input and output tensors by a host framework, or a service whose
 // device memory is owned by a framework pool it has no handle to.  They cannot provide
-// the small workspace hscale_rtn_scales needs for its amax word.  This entry point keeps
-// that word in a fixed array of this file that lives in every GPU's memory from the
+// the small workspace hscale_rtn_scales needs for its blocks' maxima.  This entry point keeps
+// them in a fixed array of this file that lives in every GPU's memory from the
 // moment the library is loaded there until the process exits.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -64,7 +64,7 @@ constexpr int kMaxDevices = 64;
 // first call in that context (with that device current) and cached per device together
 // with the context's id: a call in a new context of the same device (after
 // cudaDeviceReset) resolves it again instead of using a stale address.
-cudaError_t scratch_address(uint32_t** out) {
+cudaError_t scratch_address(void** out) {
   static std::mutex mu;
   static void* addr[kMaxDevices] = {nullptr};
   static unsigned long long ctx_of[kMaxDevices] = {0};
@@ -89,7 +89,7 @@ cudaError_t scratch_address(uint32_t** out) {
     addr[dev] = p;
     ctx_of[dev] = id;
   }
-  *out = static_cast<uint32_t*>(addr[dev]);
+  *out = addr[dev];
   return cudaSuccess;
 }
 
@@ -106,13 +106,10 @@ extern "C" int hscale_rtn_scales_noalloc(const void* w_bf16, int64_t m, int64_t 
   // the work needs hscale_rtn_workspace_bytes() of scratch, which does not depend on m or n;
   // refuse if it ever outgrows the fixed array
   if (hscale_rtn_workspace_bytes() > (size_t)HSCALE_NOALLOC_SCRATCH_BYTES) return HSCALE_ERR_WORKSPACE;
-  uint32_t* amax = nullptr;
-  if (scratch_address(&amax) != cudaSuccess) return HSCALE_ERR_CUDA;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the amax word keeps the previous call's value: clear it first
-  if (cudaMemsetAsync(amax, 0, sizeof(uint32_t), s) != cudaSuccess) return HSCALE_ERR_CUDA;
-  if (hscale::launch_amax(w_bf16, m * n, amax, s) != cudaSuccess) return HSCALE_ERR_CUDA;
-  return hscale::launch_rtn_codes(w_bf16, m, n, amax, global_scale, codes, s) == cudaSuccess
+  void* scratch = nullptr;
+  if (scratch_address(&scratch) != cudaSuccess) return HSCALE_ERR_CUDA;
+  return hscale::launch_rtn_scales(w_bf16, m, n, scratch, global_scale, codes, static_cast<cudaStream_t>(stream)) ==
+                 cudaSuccess
              ? HSCALE_OK
              : HSCALE_ERR_CUDA;
 }

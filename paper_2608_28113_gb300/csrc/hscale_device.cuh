@@ -26,12 +26,47 @@ __device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
   return r;
 }
 
+// The same, kept in its place: several of these in a row are all in flight at once (the compiler
+// otherwise moves each load down to its use).
+__device__ __forceinline__ uint4 ld_stream_v4_ahead(const void* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p));
+  return r;
+}
+
 __device__ __forceinline__ uint4 ld_nc_v4(const void* p) {
   uint4 r;
   asm("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
       : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
       : "l"(p));
   return r;
+}
+
+// 32 bytes (a group's 16 bf16 values) by one thread: one 32-byte load where the base is 32-byte
+// aligned (kWide), else two 16-byte loads, each of which uses half of every sector it touches.
+template <bool kWide>
+__device__ __forceinline__ void ld_stream_32(const uint4* p, uint4& a, uint4& b) {
+  if (kWide) {
+    asm("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
+  } else {
+    a = ld_stream_v4(p);
+    b = ld_stream_v4(p + 1);
+  }
+}
+template <bool kWide>
+__device__ __forceinline__ void st_32(uint4* p, const uint4& a, const uint4& b) {
+  if (kWide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+  } else {
+    p[0] = a;
+    p[1] = b;
+  }
 }
 
 // ---------------------------------------------------------------- bf16

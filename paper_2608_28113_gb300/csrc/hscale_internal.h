@@ -28,9 +28,13 @@ cudaError_t launch_sum_partials(const float* partials, int64_t parts, int64_t n,
 // amax over W into *amax_bits (16-bit |bf16| pattern, zero-extended); *amax_bits must be 0.
 cudaError_t launch_amax(const void* w, int64_t count, uint32_t* amax_bits, cudaStream_t stream);
 
-// s_g from *amax_bits into *global_scale, and (if codes != nullptr) the RTN codes.
-cudaError_t launch_rtn_codes(const void* w, int64_t m, int64_t n, const uint32_t* amax_bits,
-                             float* global_scale, uint8_t* codes, cudaStream_t stream);
+// s_g of *amax_bits into *global_scale.
+cudaError_t launch_scale_from_amax(const uint32_t* amax_bits, float* global_scale, cudaStream_t stream);
+
+// s_g of W into *global_scale, and (if codes != nullptr) the RTN codes; m, n > 0; workspace: 256
+// bytes, 4-byte aligned, whatever they hold.
+cudaError_t launch_rtn_scales(const void* w, int64_t m, int64_t n, void* workspace, float* global_scale,
+                              uint8_t* codes, cudaStream_t stream);
 
 // W [m, n] with rows ld_w elements apart (ld_w % 8 == 0), initial codes with rows ld_init
 // bytes apart, codes with rows ld_codes bytes apart, nibbles with rows ld_packed bytes

@@ -213,6 +213,37 @@ def test_rtn_scales_match_oracle_bit_exact():
         assert np.array_equal(codes.cpu().numpy(), oracle.rtn_codes(bits(w), s_ref))
 
 
+@pytest.mark.parametrize("m,n", [(1, 16), (7, 48), (129, 1040), (1024, 1024), (1025, 1024), (700, 8192)])
+@pytest.mark.parametrize("shift", [0, 8])
+def test_streaming_passes_over_sizes_and_alignments(m, n, shift):
+    """Global scale (alone and with the codes), RTN codes, packing and the residual around the
+    sizes where their launches change (the one-launch global scale ends at 2^20 weights; one
+    block, a few, all), from a base that is 32-byte aligned and one that is only 16-byte
+    aligned; the workspace's contents do not matter."""
+    w = wl.weight(m, n, 0.02, 3 * m + n)
+    wb = bits(w)
+    flat = torch.zeros(m * n + 16, dtype=torch.bfloat16, device=dev())
+    wd = flat[shift:shift + m * n].view(m, n)
+    wd.copy_(w)
+    s_ref, _ = oracle.global_scale(wb)
+    ws = torch.full((hs.hscale_rtn_workspace_bytes(),), 0xFF, dtype=torch.uint8, device=dev())
+    only = torch.zeros(1, dtype=torch.float32, device=dev())
+    hs.hscale_rtn_scales(wd, only, None, ws)
+    sg, codes = gpu_rtn(wd)
+    assert only.item() == float(s_ref) and sg.item() == float(s_ref)
+    c_ref = oracle.rtn_codes(wb, s_ref)
+    assert np.array_equal(codes.cpu().numpy(), c_ref)
+    packed = torch.empty(m, n // 2, dtype=torch.uint8, device=dev())
+    hs.hscale_pack_nvfp4(wd, sg, codes, packed)
+    torch.cuda.synchronize()
+    p_ref = oracle.pack(wb, s_ref, c_ref)
+    assert np.array_equal(packed.cpu().numpy(), p_ref)
+    dw = gpu_residual(wd, sg, c_ref, p_ref).double().cpu().numpy()
+    n_pad = hs.residual_ld(n) // 2
+    ref = oracle.dequant_residual(wb, s_ref, c_ref, p_ref)
+    assert np.all(np.abs(dw[:, :n] + dw[:, n_pad:n_pad + n] - ref) <= 2.0 ** -17 * np.abs(ref) + 1e-45)
+
+
 def exact_tie_matrix():
     """Groups whose max sits exactly on each E4M3 ladder value and midpoint, under
     s_g = 2^-10 (amax = 2688 * 2^-10): RTN ties are decided by round-half-even."""
