@@ -7,7 +7,7 @@
 //                       (Eqs. 8-11) is scored by sum_j h_j (|w_j| - s q_j)^2 (Eqs. 6, 12,
 //                       13); the best code is re-quantized exactly and packed.  Their
 //                       4over6 instances decide Algorithm 2's initial code in place.  One
-//                       per-group body (search_unit) under four deals of the units:
+//                       per-group body (search_unit) under five deals of the units:
 //                         refine_kernel         2-D views, ragged rows (static)
 //                         refine_linear_kernel  contiguous W, static (a search beside
 //                                               another kernel, or a tiny one)
@@ -15,6 +15,8 @@
 //                                               SM, units shared through shared memory
 //                         refine_shared_kernel  contiguous W, long searches: units shared
 //                                               through a counter in a caller workspace
+//                         refine_flat_kernel    2-D views and ragged rows alone on the GPU: as
+//                                               refine_sm_kernel, over flattened groups
 //   fourover6_codes_kernel  Algorithm 2's initial codes as a separate pass
 //   pack_kernel         exact FP4 quantization with given codes (Eq. 2)
 //
@@ -496,13 +498,13 @@ __device__ __forceinline__ SearchConsts search_consts(const ScaleDomain& d, bool
   return k;
 }
 
-// One unit of the contiguous layout: every lane searches its group g (index `go`, whose 16
-// bf16 values are p, q and sit at wg in W; h slice hv2 of column group hcol = chunk * 32 +
-// lane) and writes code byte go and nibble word go.  All 32 lanes take part (the warp
-// rescores ambiguous groups together).
+// One unit: every lane searches its group, whose 16 bf16 values are p, q and sit at wg in W, with the
+// h slice hv2 (its sum hsum) of column group hcol, and writes code byte oc and nibble word op
+// (initial code byte oi).  All 32 lanes take part (the warp rescores ambiguous groups together); a
+// lane that is not `active` writes nothing.
 template <bool kFourOverSix>
-__device__ __forceinline__ void search_unit(const uint4& p, const uint4& q, const uint4* wg, int64_t go, int64_t chunk,
-                                            const float2 (&hv2)[8], float hsum, const uint4* __restrict__ w,
+__device__ __forceinline__ void search_unit(const uint4& p, const uint4& q, const uint4* wg, int64_t oi, int64_t oc,
+                                            int64_t op, int64_t hcol, bool active, const float2 (&hv2)[8], float hsum,
                                             const float* __restrict__ h, const float4* tab, const ScaleDomain& d,
                                             const SearchConsts& k, const uint8_t* init_codes, int down, int up,
                                             uint8_t* codes_out, uint2* __restrict__ packed_out) {
@@ -512,7 +514,7 @@ __device__ __forceinline__ void search_unit(const uint4& p, const uint4& q, cons
   unpack_group(p, q, d.pw, G);
   int c0;
   if (!kFourOverSix && init_codes != nullptr) {
-    c0 = init_codes[go] & 0x7F;
+    c0 = init_codes[oi] & 0x7F;
     c0 = c0 < 1 ? 1 : (c0 > (int)kE4M3MaxCode ? (int)kE4M3MaxCode : c0);
   } else {
     c0 = kFourOverSix ? fourover6_init_code(G, wg, tab, amax_k, d.sgk, d.pw, k.inv4, k.inv6, k.b4, k.b6)
@@ -527,32 +529,33 @@ __device__ __forceinline__ void search_unit(const uint4& p, const uint4& q, cons
 
   // the cheap sufficient test with the loose energy bound first; the exact energy and the
   // full test only for the groups it cannot clear
-  bool ambiguous = hi > lo && !fast_winner_clear(e1, e2, energy_bound(hsum, amax_k));
+  bool ambiguous = active && hi > lo && !fast_winner_clear(e1, e2, energy_bound(hsum, amax_k));
   if (ambiguous) ambiguous = !fast_winner_certain(e1, e2, group_energy(G, hv2));
   unsigned amb = __ballot_sync(0xFFFFFFFFu, ambiguous);
   while (amb) {
     const int owner = __ffs(amb) - 1;
     amb &= amb - 1;
-    const int64_t g_own = __shfl_sync(0xFFFFFFFFu, go, owner);
+    const uint16_t* wg_own = reinterpret_cast<const uint16_t*>(
+        __shfl_sync(0xFFFFFFFFu, (unsigned long long)reinterpret_cast<uintptr_t>(wg), owner));
+    const int64_t hcol_own = __shfl_sync(0xFFFFFFFFu, (int)hcol, owner);
     const int c0o = __shfl_sync(0xFFFFFFFFu, c0, owner);
     const int loo = __shfl_sync(0xFFFFFFFFu, lo, owner);
     const int hio = __shfl_sync(0xFFFFFFFFu, hi, owner);
-    const int bc = warp_exact_search(reinterpret_cast<const uint16_t*>(w) + g_own * 16, h,
-                                     chunk * 32 + owner, c0o, loo, hio, d.sgk, d.pw);
+    const int bc = warp_exact_search(wg_own, h, hcol_own, c0o, loo, hio, d.sgk, d.pw);
     if (lane == owner) best = bc;
   }
 
-  codes_out[go] = (uint8_t)best;
+  if (!active) return;
+  codes_out[oc] = (uint8_t)best;
   if (packed_out != nullptr)
-    packed_out[go] = quantize_pack(G, (uint32_t)best, tab[best].z, d.sgk, d.pw,
+    packed_out[op] = quantize_pack(G, (uint32_t)best, tab[best].z, d.sgk, d.pw,
                                    reinterpret_cast<const uint16_t*>(wg));
 }
 
-// Loads the h slice of column chunk `chunk` (this lane's 16 values) and its sum.
-__device__ __forceinline__ void load_h_slice(const float* __restrict__ h, int64_t chunk, float2 (&hv2)[8],
+// Loads the h slice of column group hcol (16 values) and its sum.
+__device__ __forceinline__ void load_h_slice(const float* __restrict__ h, int64_t hcol, float2 (&hv2)[8],
                                              float& hsum) {
-  const int lane = threadIdx.x & 31;
-  const float4* hp = reinterpret_cast<const float4*>(h + (chunk * 32 + lane) * 16);
+  const float4* hp = reinterpret_cast<const float4*>(h + hcol * 16);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const float4 t = hp[i];
@@ -582,7 +585,8 @@ refine_linear_kernel(const uint4* __restrict__ w, const float* __restrict__ h, i
   __shared__ float4 tab[128];
   __shared__ __align__(16) uint4 stage[kWarpsPerRefineBlock][2][64];
   const ScaleDomain d = make_scale_domain(*global_scale);
-  const SearchConsts k = search_consts(d, kFourOverSix);
+  __shared__ SearchConsts k;  // read per unit: in registers the 4over6 instance would spill more
+  if (threadIdx.x == 0) k = search_consts(d, kFourOverSix);
   for (int c = threadIdx.x; c < 128; c += blockDim.x) tab[c] = candidate_constants((uint32_t)c, d.sgk);
 
   // this lane's group of unit u: uint4 words 64 u + 2 lane and the one after
@@ -621,13 +625,13 @@ refine_linear_kernel(const uint4* __restrict__ w, const float* __restrict__ h, i
 
     if (h != nullptr && chunk != cur_chunk) {
       cur_chunk = chunk;
-      load_h_slice(h, chunk, hv2, hsum);
+      load_h_slice(h, (int64_t)chunk * 32 + lane, hv2, hsum);
     }
 
     cp_async_wait_1();  // this lane's copy of the current unit has landed
     const uint4* cur = buf ? st1 : st0;
-    search_unit<kFourOverSix>(cur[0], cur[32], wp, go, chunk, hv2, hsum, w, h, tab, d, k, init_codes, down, up,
-                              codes_out, packed_out);
+    search_unit<kFourOverSix>(cur[0], cur[32], wp, go, go, go, (int64_t)chunk * 32 + lane, true, hv2, hsum, h, tab, d,
+                              k, init_codes, down, up, codes_out, packed_out);
     wp += wstep;
     go += ostep;
     chunk += chunk_step;
@@ -661,7 +665,8 @@ refine_shared_kernel(const uint4* __restrict__ w, const float* __restrict__ h, u
   __shared__ float4 tab[128];
   __shared__ __align__(16) uint4 stage[kWarpsPerRefineBlock][2][64];
   const ScaleDomain d = make_scale_domain(*global_scale);
-  const SearchConsts k = search_consts(d, kFourOverSix);
+  __shared__ SearchConsts k;  // read per unit: in registers the 4over6 instance would spill more
+  if (threadIdx.x == 0) k = search_consts(d, kFourOverSix);
   for (int c = threadIdx.x; c < 128; c += blockDim.x) tab[c] = candidate_constants((uint32_t)c, d.sgk);
 
   // the current unit v = (row, chunk) and the end of its batch; lane 0 holds the index of
@@ -717,13 +722,14 @@ refine_shared_kernel(const uint4* __restrict__ w, const float* __restrict__ h, u
 
     if (h != nullptr && chunk != cur_chunk) {
       cur_chunk = chunk;
-      load_h_slice(h, chunk, hv2, hsum);
+      load_h_slice(h, (int64_t)chunk * 32 + lane, hv2, hsum);
     }
 
     cp_async_wait_1();  // this lane's copy of the current unit has landed
     const uint4* cur = buf ? st1 : st0;
-    search_unit<kFourOverSix>(cur[0], cur[32], group_of(row, chunk), (int64_t)row * ng + (int64_t)chunk * 32 + lane,
-                              chunk, hv2, hsum, w, h, tab, d, k, init_codes, down, up, codes_out, packed_out);
+    const int64_t go = (int64_t)row * ng + (int64_t)chunk * 32 + lane;
+    search_unit<kFourOverSix>(cur[0], cur[32], group_of(row, chunk), go, go, go, (int64_t)chunk * 32 + lane, true, hv2,
+                              hsum, h, tab, d, k, init_codes, down, up, codes_out, packed_out);
     v = v2;
     row = row2;
     chunk = chunk2;
@@ -754,7 +760,8 @@ refine_sm_kernel(const uint4* __restrict__ w, const float* __restrict__ h, uint3
   __shared__ __align__(16) uint4 stage[kSmWarps][2][64];
   __shared__ unsigned next_unit;
   const ScaleDomain d = make_scale_domain(*global_scale);
-  const SearchConsts k = search_consts(d, kFourOverSix);
+  __shared__ SearchConsts k;  // read per unit: in registers the 4over6 instance would spill more
+  if (threadIdx.x == 0) k = search_consts(d, kFourOverSix);
   for (int c = threadIdx.x; c < 128; c += blockDim.x) tab[c] = candidate_constants((uint32_t)c, d.sgk);
 
   // this CTA's units [vbeg, vlim); unit v is row v % m of column chunk v / m
@@ -803,16 +810,97 @@ refine_sm_kernel(const uint4* __restrict__ w, const float* __restrict__ h, uint3
 
     if (h != nullptr && chunk != cur_chunk) {
       cur_chunk = chunk;
-      load_h_slice(h, chunk, hv2, hsum);
+      load_h_slice(h, (int64_t)chunk * 32 + lane, hv2, hsum);
     }
 
     cp_async_wait_1();  // this lane's copy of the current unit has landed
     const uint4* cur = buf ? st1 : st0;
-    search_unit<kFourOverSix>(cur[0], cur[32], group_of(row, chunk), (int64_t)row * ng + (int64_t)chunk * 32 + lane,
-                              chunk, hv2, hsum, w, h, tab, d, k, init_codes, down, up, codes_out, packed_out);
+    const int64_t go = (int64_t)row * ng + (int64_t)chunk * 32 + lane;
+    search_unit<kFourOverSix>(cur[0], cur[32], group_of(row, chunk), go, go, go, (int64_t)chunk * 32 + lane, true, hv2,
+                              hsum, h, tab, d, k, init_codes, down, up, codes_out, packed_out);
     v = v2;
     row = row2;
     chunk = chunk2;
+    buf ^= 1;
+  }
+}
+
+// The same schedule for every other layout: rows that are not whole 32-group chunks, and 2-D
+// views.  A unit is 32 consecutive groups of the flattened (row, column group) order, so only
+// the last unit has idle lanes however short the rows are (a unit per row chunk leaves 10 % idle
+// at 201 groups a row, 45 % at 35); each lane divides out its own row and column and loads its own
+// h slice per unit (from L1: about 30 of a unit's 900 instructions).  One GB300, 3001 x 3216 with
+// the 4over6 start, global scale included: 43.1 -> 39.4 us against the static deal of row chunks
+// (refine_kernel); 20000 x 560, 16 candidates: 87.7 -> 52.2 us.
+template <bool kFourOverSix>
+__global__ void __launch_bounds__(kSmWarps * 32, 1)
+refine_flat_kernel(const uint4* __restrict__ w, int64_t row_words, const float* __restrict__ h, uint32_t groups,
+                   uint32_t ng, const float* __restrict__ global_scale, const uint8_t* init_codes, int64_t ld_i,
+                   int down, int up, uint8_t* codes_out, int64_t ld_c, uint2* __restrict__ packed_out, int64_t ld_p) {
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  __shared__ float4 tab[128];
+  __shared__ __align__(16) uint4 stage[kSmWarps][2][64];
+  __shared__ unsigned next_unit;
+  const ScaleDomain d = make_scale_domain(*global_scale);
+  __shared__ SearchConsts k;  // read per unit: in registers the 4over6 instance would spill more
+  if (threadIdx.x == 0) k = search_consts(d, kFourOverSix);
+  for (int c = threadIdx.x; c < 128; c += blockDim.x) tab[c] = candidate_constants((uint32_t)c, d.sgk);
+
+  // this CTA's units [vbeg, vlim)
+  const uint32_t units = (groups + 31) / 32;
+  const uint32_t vbeg = (uint32_t)(((uint64_t)units * blockIdx.x) / gridDim.x);
+  const uint32_t vlim = (uint32_t)(((uint64_t)units * (blockIdx.x + 1)) / gridDim.x);
+  if (threadIdx.x == 0) next_unit = vbeg + kSmWarps;  // the first kSmWarps units go to warps in order
+  // a lane past the last group searches that group again and writes nothing
+  auto locate = [&](uint32_t v, uint32_t& row, uint32_t& col) {
+    const uint32_t g = min(32 * v + lane, groups - 1);
+    row = g / ng;
+    col = g - row * ng;
+  };
+  auto group_of = [&](uint32_t row, uint32_t col) { return w + (int64_t)row * row_words + 2 * (int64_t)col; };
+  uint4* const st0 = &stage[warp][0][lane];
+  uint4* const st1 = &stage[warp][1][lane];
+  uint32_t v = vbeg + warp, row = 0, col = 0;
+  if (v < vlim) {
+    locate(v, row, col);
+    const uint4* s = group_of(row, col);
+    cp_async16(st0, s);
+    cp_async16(st0 + 32, s + 1);
+  }
+  cp_async_commit();
+  __syncthreads();  // the candidate table and the counter
+
+  float2 hv2[8];
+  float hsum = 16.0f;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) hv2[j] = make_float2(1.0f, 1.0f);
+
+  int buf = 0;
+  while (v < vlim) {
+    uint32_t v2 = 0;
+    if (lane == 0) v2 = atomicAdd(&next_unit, 1u);
+    v2 = __shfl_sync(0xFFFFFFFFu, v2, 0);
+    uint32_t row2 = 0, col2 = 0;
+    if (v2 < vlim) {
+      locate(v2, row2, col2);
+      uint4* dst = buf ? st0 : st1;
+      const uint4* s = group_of(row2, col2);
+      cp_async16(dst, s);
+      cp_async16(dst + 32, s + 1);
+    }
+    cp_async_commit();
+
+    if (h != nullptr) load_h_slice(h, col, hv2, hsum);
+
+    cp_async_wait_1();  // this lane's copy of the current unit has landed
+    const uint4* cur = buf ? st1 : st0;
+    search_unit<kFourOverSix>(cur[0], cur[32], group_of(row, col), row * ld_i + col, row * ld_c + col, row * ld_p + col,
+                              col, 32 * v + lane < groups, hv2, hsum, h, tab, d, k, init_codes, down, up, codes_out,
+                              packed_out);
+    v = v2;
+    row = row2;
+    col = col2;
     buf ^= 1;
   }
 }
@@ -1025,6 +1113,22 @@ cudaError_t launch_refine(const void* w, int64_t ld_w, const float* h, int64_t m
                                                          global_scale, fourover6 ? nullptr : init_codes, down, up,
                                                          codes_out, reinterpret_cast<uint2*>(packed_out));
     return cudaGetLastError();
+  }
+  // any other layout alone on the GPU, from two units per warp on: the same schedule over the
+  // flattened groups; smaller searches spread better as 4-warp CTAs
+  const int64_t groups = m * ng;
+  if (ctas_per_sm == 0 && groups < (int64_t(1) << 31) && groups >= 64 * (int64_t)info.sm_count * kSmWarps) {
+    auto fk = fourover6 ? refine_flat_kernel<true> : refine_flat_kernel<false>;
+    const int fits = fourover6 ? occupancy_blocks<refine_flat_kernel<true>>(kSmWarps * 32)
+                               : occupancy_blocks<refine_flat_kernel<false>>(kSmWarps * 32);
+    if (fits >= 1) {
+      fk<<<(unsigned)info.sm_count, kSmWarps * 32, 0, stream>>>(static_cast<const uint4*>(w), ld_w / 8, h,
+                                                               (uint32_t)groups, (uint32_t)ng, global_scale,
+                                                               fourover6 ? nullptr : init_codes, ld_init, down, up,
+                                                               codes_out, ld_codes, reinterpret_cast<uint2*>(packed_out),
+                                                               ld_packed / 8);
+      return cudaGetLastError();
+    }
   }
   auto kernel = fourover6 ? refine_kernel<true> : refine_kernel<false>;
   kernel<<<(unsigned)blocks, kRefineThreads, 0, stream>>>(static_cast<const uint4*>(w), ld_w, h, m, ng, global_scale,

@@ -845,6 +845,44 @@ def test_strided_column_blocks_match_whole_matrix(init):
                    f"strided block {c0}:{c1}, init {init}")
 
 
+@pytest.mark.parametrize("m,n,pad", [(20001, 240, 0), (3001, 1616, 0), (4300, 1024, 48), (90000, 48, 16)])
+@pytest.mark.parametrize("init", ["rtn", "given", "4over6"])
+def test_flat_schedule_matches_the_static_deal(m, n, pad, init):
+    """Searches of ragged rows and of views, large enough for the schedule over flattened groups
+    (ctas_per_sm = 0), write the bytes of the static deal (ctas_per_sm = 7), nothing outside the
+    view, and the oracle's codes on the first and last rows."""
+    wide = torch.zeros(m, n + 2 * pad, dtype=torch.bfloat16, device=dev())
+    wide[:, pad:pad + n] = wl.weight(m, n, 0.02, m + n, device=dev())
+    w = wide[:, pad:pad + n]
+    h = torch.rand(n, device=dev()) + 0.01
+    sg = (w.float().abs().max() / 2688).view(1).contiguous()
+    g = torch.Generator(device=dev()).manual_seed(m)
+    init_codes = torch.randint(1, 127, (m, n // 16), generator=g, device=dev(), dtype=torch.uint8) if init == "given" else None
+    out = []
+    for ctas in (0, 7):
+        codes = torch.full((m, (n + 2 * pad) // 16), 0xEE, dtype=torch.uint8, device=dev())
+        packed = torch.full((m, (n + 2 * pad) // 2), 0xEE, dtype=torch.uint8, device=dev())
+        hs.hscale_refine_scales_strided(w, h, sg, init_codes, init == "4over6", 4, 4, codes[:, pad // 16:(pad + n) // 16],
+                                        packed[:, pad // 2:(pad + n) // 2], ctas)
+        torch.cuda.synchronize()
+        out.append((codes, packed))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    if pad:
+        assert bool((out[0][0][:, :pad // 16] == 0xEE).all()) and bool((out[0][1][:, (pad + n) // 2:] == 0xEE).all())
+    rows = torch.cat([torch.arange(8), torch.arange(m - 8, m)]).to(dev())
+    wb = bits(w[rows].contiguous().cpu())
+    s_ref = np.float32(sg.item())
+    first, anchor_tie = None, False
+    if init == "given":
+        first = init_codes[rows].cpu().numpy()
+    elif init == "4over6":
+        first, anchor_tie = oracle.fourover6_codes(wb, s_ref)
+        anchor_tie = anchor_tie.astype(bool)
+    ref = oracle.refine(wb, h.cpu().numpy(), s_ref, first, 4, 4)
+    got = out[0][0][rows][:, pad // 16:(pad + n) // 16].cpu().numpy()
+    assert not np.any((got != ref["codes"]) & ~ref["near_tie"].astype(bool) & ~anchor_tie)
+
+
 def test_strided_row_slice_and_no_packed_output():
     """A row slice (one row of a larger matrix) and a view without nibbles."""
     m, n = 40, 1024
