@@ -161,9 +161,10 @@ template <int kMode>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
             int kb_half, int tiles_n, int tiles_total,
-            double* __restrict__ partials, float* __restrict__ H, int64_t h_rows, int64_t h_cols, int64_t ld_h) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+            double* __restrict__ partials, float* __restrict__ H, int64_t h_rows, int64_t h_cols, int64_t ld_h,
+            int grouped) {
+  extern __shared__ __align__(16) uint8_t dynamic_smem[];
+  uint8_t* smem = dynamic_smem + ((1024u - (smem_addr(dynamic_smem) & 1023u)) & 1023u);
   uint8_t* tile_a = smem;
   uint8_t* tile_b = smem + kStages * kTileABytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
@@ -180,7 +181,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   // squares.  The Hessian modes take one tile per CTA.
   constexpr bool kPersistent = kMode == 0;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int ntiles = kPersistent ? (tiles_total - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 1;
   const int tile_m = blockIdx.x / tiles_n, tile_n = blockIdx.x - tile_m * tiles_n;
   constexpr bool kAccum = kMode != 0;
@@ -208,93 +209,98 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  const uint32_t tmem_d = *tmem_slot;
+  const uint32_t tmem_d = warp_uniform(*tmem_slot);
   if (warp == 0) {
-    if (lane == 0) {
-      uint64_t policy;
-      asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(policy));
-      bool go = true;
-      for (int i = 0; i < ntiles && go; ++i) {
-        const int t = (int)blockIdx.x + i * (int)gridDim.x;
-        int tm = t / tiles_n, tn = t - tm * tiles_n;
-        if (kMode == 0) raster_tile(t, tiles_n, tiles_total, tm, tn);
-        for (int kb = 0; kb < kb_total; ++kb) {
-          // the ring's position counts K blocks over all of the CTA's tiles
-          const int g = i * kb_total + kb;
-          const int s = g % kStages;
-          const uint32_t round = (uint32_t)(g / kStages);
-          if (!mbar_wait(&empty[s], (round & 1u) ^ 1u)) {
-            atomicOr(failed, 1u);
-            go = false;
-            break;
-          }
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(policy));
+    uint32_t s = 0, parity = 1;  // the ring's position, over all of the CTA's tiles
+    bool go = true;
+    for (int i = 0; i < ntiles && go; ++i) {
+      const int t = (int)blockIdx.x + i * (int)gridDim.x;
+      int tm = t / tiles_n, tn = t - tm * tiles_n;
+      if (kMode == 0) raster_tile(t, tiles_n, tiles_total, tm, tn);
+      for (int kb = 0; kb < kb_total; ++kb) {
+        if (!mbar_wait_warp(&empty[s], parity)) {
+          if (lane == 0) atomicOr(failed, 1u);
+          go = false;
+          break;
+        }
+        if (elect_one()) {
           mbar_arrive_expect_tx(&full[s], kStageBytes);
-          if (kMode == 3) {
+          uint8_t* a = tile_a + s * kTileABytes;
+          uint8_t* b = tile_b + s * kTileBBytes;
+          if (kMode == 3 && grouped) {
+            // boxes of two and four 64-channel groups
+            tma_load_3d(a, &xmap, 0, kb * kBK, tm * (kBM / 64), &full[s], policy);
+            tma_load_3d(b, &wmap, 0, kb * kBK, tn * (kBN / 64), &full[s], policy);
+          } else if (kMode == 3) {
 #pragma unroll
             for (int j = 0; j < kBM / 64; ++j)
-              tma_load_2d(tile_a + s * kTileABytes + j * kBoxBytes, &xmap, tm * kBM + 64 * j, kb * kBK, &full[s],
-                          policy);
+              tma_load_2d(a + j * kBoxBytes, &xmap, tm * kBM + 64 * j, kb * kBK, &full[s], policy);
 #pragma unroll
             for (int j = 0; j < kBN / 64; ++j)
-              tma_load_2d(tile_b + s * kTileBBytes + j * kBoxBytes, &wmap, tn * kBN + 64 * j, kb * kBK, &full[s],
-                          policy);
+              tma_load_2d(b + j * kBoxBytes, &wmap, tn * kBN + 64 * j, kb * kBK, &full[s], policy);
           } else {
             const int xk = (kAccum || kb < kb_half ? kb : kb - kb_half) * kBK;
-            tma_load_2d(tile_a + s * kTileABytes, &xmap, xk, tm * kBM, &full[s], policy);
-            tma_load_2d(tile_b + s * kTileBBytes, &wmap, kb * kBK, tn * kBN, &full[s], policy);
+            tma_load_2d(a, &xmap, xk, tm * kBM, &full[s], policy);
+            tma_load_2d(b, &wmap, kb * kBK, tn * kBN, &full[s], policy);
           }
+        }
+        __syncwarp();
+        if (++s == kStages) {
+          s = 0;
+          parity ^= 1u;
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // segments of kSegBlocks K blocks, each accumulated from zero
-      const int nseg = (kb_total + kSegBlocks - 1) / kSegBlocks;
-      bool ok = true;
-      for (int i = 0; i < ntiles && ok; ++i) {
-        for (int seg = 0; seg < nseg && ok; ++seg) {
-          // the previous segment's partial (of this tile or the one before) must have been
-          // read out of TMEM
-          const int gs = i * nseg + seg;
-          if (gs >= 1 && !mbar_wait(seg_empty, (uint32_t)(gs - 1) & 1u)) {
-            atomicOr(failed, 1u);
+    // segments of kSegBlocks K blocks, each accumulated from zero
+    const int nseg = (kb_total + kSegBlocks - 1) / kSegBlocks;
+    uint32_t s = 0, parity = 0, gs = 0;  // gs counts the segments over all of the CTA's tiles
+    bool ok = true;
+    for (int i = 0; i < ntiles && ok; ++i) {
+      for (int seg = 0; seg < nseg && ok; ++seg, ++gs) {
+        // the previous segment's partial (of this tile or the one before) must have been
+        // read out of TMEM
+        if (gs >= 1 && !mbar_wait_warp(seg_empty, (gs - 1) & 1u)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const int kb0 = seg * kSegBlocks, kb1 = min(kb_total, kb0 + kSegBlocks);
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!mbar_wait_warp(&full[s], parity)) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          const uint32_t d = tmem_d;
-          const int kb0 = seg * kSegBlocks, kb1 = min(kb_total, kb0 + kSegBlocks);
-          for (int kb = kb0; kb < kb1; ++kb) {
-            const int g = i * kb_total + kb;
-            const int s = g % kStages;
-            const uint32_t round = (uint32_t)(g / kStages);
-            if (!mbar_wait(&full[s], round & 1u)) {
-              atomicOr(failed, 1u);
-              ok = false;
-              break;
-            }
-            tc_fence_after_sync();
+          if (elect_one()) {
+            const uint32_t a = smem_addr(tile_a + s * kTileABytes), b = smem_addr(tile_b + s * kTileBBytes);
             if (kMode == 3) {
               // MN-major: 16 K rows are two 1024-byte swizzle atoms further
-              const uint64_t ad = smem_desc_mn_sw128(smem_addr(tile_a + s * kTileABytes), kBoxBytes);
-              const uint64_t bd = smem_desc_mn_sw128(smem_addr(tile_b + s * kTileBBytes), kBoxBytes);
+              const uint64_t ad = smem_desc_mn_sw128(a, kBoxBytes), bd = smem_desc_mn_sw128(b, kBoxBytes);
 #pragma unroll
               for (int kk = 0; kk < kBK / 16; ++kk)
-                umma_bf16(d, ad + 128 * kk, bd + 128 * kk, kIdescMN, (uint32_t)(kb > kb0 || kk > 0));
+                umma_bf16(tmem_d, ad + 128 * kk, bd + 128 * kk, kIdescMN, (uint32_t)(kb > kb0 || kk > 0));
             } else {
-              const uint64_t ad = smem_desc_k_sw128(smem_addr(tile_a + s * kTileABytes));
-              const uint64_t bd = smem_desc_k_sw128(smem_addr(tile_b + s * kTileBBytes));
+              const uint64_t ad = smem_desc_k_sw128(a), bd = smem_desc_k_sw128(b);
 #pragma unroll
               for (int kk = 0; kk < kBK / 16; ++kk)
-                umma_bf16(d, ad + 2 * kk, bd + 2 * kk, kIdesc, (uint32_t)(kb > kb0 || kk > 0));
+                umma_bf16(tmem_d, ad + 2 * kk, bd + 2 * kk, kIdesc, (uint32_t)(kb > kb0 || kk > 0));
             }
             umma_commit(smem_addr(&empty[s]));
+            // fires once every MMA issued above has completed
+            if (kb + 1 == kb1) umma_commit(smem_addr(seg_full));
           }
-          // fires once every MMA issued above has completed
-          if (ok) umma_commit(smem_addr(seg_full));
+          __syncwarp();
+          if (++s == kStages) {
+            s = 0;
+            parity ^= 1u;
+          }
         }
       }
     }
+    if (!ok && lane == 0) atomicOr(failed, 1u);
     __syncwarp();
   } else {
     // epilogue warps 2-9: TMEM lane quarter warp % 4 (a warp may only touch that quarter),
@@ -414,21 +420,33 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   }
 }
 
-// X [tokens, n] (row stride ld_x) -> Xt [n, tokens] (row stride ld_t), 32 x 32 tiles
-// through shared memory so both the reads and the writes are coalesced.
+// X [tokens, n] (row stride ld_x, 2-byte aligned) -> Xt [n, tokens] (row stride ld_t, a multiple of
+// 8), 64 x 64 tiles through shared memory: the reads run along channels, two bytes a lane (rows
+// may start anywhere), the writes along tokens, eight bytes a thread (32 x 32 tiles with two-byte
+// writes took 130 us for 16384 x 4095, now 57).
 __global__ void __launch_bounds__(256) transpose_kernel(const uint16_t* __restrict__ x, int64_t tokens, int64_t n,
                                                         int64_t ld_x, uint16_t* __restrict__ xt, int64_t ld_t) {
-  __shared__ uint16_t tile[32][33];
-  const int64_t t0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 rows of 32 per pass
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t t = t0 + k, c = c0 + tx;
-    tile[k][tx] = (t < tokens && c < n) ? x[t * ld_x + c] : (uint16_t)0;
+  __shared__ uint16_t tile[64][66];
+  const int64_t t0 = (int64_t)blockIdx.x * 64, c0 = (int64_t)blockIdx.y * 64;
+  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;  // 4 rows of 64 per pass
+  uint16_t v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int64_t t = t0 + ty + 4 * k, c = c0 + tx;
+    v[k] = (t < tokens && c < n) ? x[t * ld_x + c] : (uint16_t)0;
   }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) tile[ty + 4 * k][tx] = v[k];
   __syncthreads();
-  for (int k = ty; k < 32; k += 8) {
-    const int64_t c = c0 + k, t = t0 + tx;
-    if (c < n && t < tokens) xt[c * ld_t + t] = tile[tx][k];
+  // four tokens of one channel each; rows of Xt reach ld_t >= tokens (its padding takes zeros)
+  const int q = 4 * (threadIdx.x & 15), cy = threadIdx.x >> 4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int cc = cy + 16 * k;
+    if (c0 + cc >= n || t0 + q >= ld_t) continue;
+    *reinterpret_cast<uint2*>(xt + (c0 + cc) * ld_t + t0 + q) =
+        make_uint2((uint32_t)tile[q][cc] | ((uint32_t)tile[q + 1][cc] << 16),
+                   (uint32_t)tile[q + 2][cc] | ((uint32_t)tile[q + 3][cc] << 16));
   }
 }
 
@@ -509,7 +527,7 @@ cudaError_t launch_output_error(const void* x, int64_t tokens, int64_t n, int64_
   if ((err = current_device_info(&info)) != cudaSuccess) return err;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(tiles, info.sm_count));
   gemm_kernel<0><<<(unsigned)grid, kGemmThreads, kGemmSmemBytes, stream>>>(
-      xmap, wmap, (int)(n_pad / kBK), (int)tiles_n, (int)tiles, partials, nullptr, 0, 0, 0);
+      xmap, wmap, (int)(n_pad / kBK), (int)tiles_n, (int)tiles, partials, nullptr, 0, 0, 0, 0);
   err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   reduce_kernel<<<1, 256, 0, stream>>>(partials, grid, out);
@@ -526,26 +544,35 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
   const int64_t tiles_n = (n + kBN - 1) / kBN;
   const int64_t tiles = ((n + kBM - 1) / kBM) * tiles_n;
   if ((reinterpret_cast<uintptr_t>(x) & 15) == 0 && ld_x % 8 == 0) {
-    // X read as it is: 64-channel x 64-token boxes, MN-major operands (kMode 3)
-    CUtensorMap map;
-    const cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)tokens};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld_x * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kBK};
-    const cuuint32_t estr[2] = {1, 1};
-    if (encode(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(x), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    // X read as it is: 64-channel x 64-token boxes, MN-major operands (kMode 3).  Where n is whole
+    // 64-channel groups, X is mapped as [n / 64][tokens][64] and one load takes an operand's two or
+    // four boxes, instead of six loads a stage; otherwise a last group would reach past the rows'
+    // ends, and each box is a load of its own, bounded by n.
+    const bool grouped = n % 64 == 0;
+    CUtensorMap map, bmap;
+    const cuuint64_t dims2[2] = {(cuuint64_t)n, (cuuint64_t)tokens};
+    const cuuint64_t strides2[1] = {(cuuint64_t)ld_x * 2};
+    const cuuint64_t dims3[3] = {64, (cuuint64_t)tokens, (cuuint64_t)(n / 64)};
+    const cuuint64_t strides3[2] = {(cuuint64_t)ld_x * 2, 128};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    auto encode_x = [&](CUtensorMap* out, cuuint32_t groups) {
+      const cuuint32_t box[3] = {64, (cuuint32_t)kBK, groups};
+      return encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, grouped ? 3 : 2, const_cast<void*>(x), grouped ? dims3 : dims2,
+                    grouped ? strides3 : strides2, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    if (encode_x(&map, kBM / 64) != CUDA_SUCCESS || encode_x(&bmap, kBN / 64) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
     err = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<3>), (int)kGemmSmemBytes);
     if (err != cudaSuccess) return err;
     gemm_kernel<3><<<(unsigned)tiles, kGemmThreads, kGemmSmemBytes, stream>>>(
-        map, map, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
+        map, bmap, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h, grouped ? 1 : 0);
     return cudaGetLastError();
   }
   // X with rows that are not 16-byte aligned: transposed first (tokens contiguous per
   // channel), then both operands K-major (kMode 1)
   const int64_t ld_t = hessian_full_ld(tokens);
-  const dim3 tgrid((unsigned)((tokens + 31) / 32), (unsigned)((n + 31) / 32));
+  const dim3 tgrid((unsigned)((tokens + 63) / 64), (unsigned)((n + 63) / 64));
   transpose_kernel<<<tgrid, 256, 0, stream>>>(static_cast<const uint16_t*>(x), tokens, n, ld_x,
                                               static_cast<uint16_t*>(xt), ld_t);
   err = cudaGetLastError();
@@ -565,7 +592,7 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
       ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<1>), (int)kGemmSmemBytes);
   if (attr_status != cudaSuccess) return attr_status;
   gemm_kernel<1><<<(unsigned)tiles, kGemmThreads, kGemmSmemBytes, stream>>>(
-      amap, bmap, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h);
+      amap, bmap, (int)((tokens + kBK - 1) / kBK), (int)tiles_n, (int)tiles, nullptr, H, n, n, ld_h, 0);
   return cudaGetLastError();
 }
 
