@@ -93,6 +93,9 @@ def library_path() -> pathlib.Path:
 def load(build_if_missing: bool = False) -> ctypes.CDLL:
     """The loaded CUDA library.  Raises if it has not been built."""
     global _lib
+    lib = _lib  # set once, complete: every later call passes without the lock
+    if lib is not None:
+        return lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -131,8 +134,14 @@ def hscale_device_error_flags() -> int:
     return int(v.value)
 
 
+# the current stream's handle without building a Stream object on every call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
