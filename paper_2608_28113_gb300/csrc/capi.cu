@@ -74,13 +74,14 @@ int hscale_abi_version(void) { return 4; }
 
 int hscale_device_error_flags(uint32_t* flags) {
   if (flags == nullptr) return HSCALE_ERR_NULL;
-  uint32_t a = 0, b = 0, c = 0, d = 0, e = 0;
+  uint32_t a = 0, b = 0, c = 0, d = 0, e = 0, f = 0;
   cudaError_t err = hscale::read_hessian_device_error(&a);
   if (err == cudaSuccess) err = hscale::read_output_error_device_error(&b);
   if (err == cudaSuccess) err = hscale::read_selftest_device_error(&c);
   if (err == cudaSuccess) err = hscale::read_update_device_error(&d);
   if (err == cudaSuccess) err = hscale::read_gptq_device_error(&e);
-  *flags = a | b | c | d | e;
+  if (err == cudaSuccess) err = hscale::read_hessian_cluster_device_error(&f);
+  *flags = a | b | c | d | e | f;
   return from_cuda(err);
 }
 

@@ -88,6 +88,14 @@ int64_t hessian_full_ld(int64_t tokens);
 cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_t ld_x, float* H, int64_t ld_h,
                                 void* xt, cudaStream_t stream);
 
+// The same by clusters of `size` CTAs per tile that split the tokens, for widths with few tiles;
+// size 1: not worth it (few 2048-token segments, or tiles enough for the SMs).  h_aligned: H's rows
+// are 16-byte aligned.  The operand maps are launch_hessian_full's.
+int hessian_cluster_size(int64_t tokens, int64_t n, bool h_aligned, int sm_count);
+cudaError_t launch_hessian_cluster(int size, const CUtensorMap& amap, const CUtensorMap& bmap, bool mn_major,
+                                   bool grouped, int64_t tokens, int64_t n, float* H, int64_t ld_h,
+                                   cudaStream_t stream);
+
 // Algorithm 3 (GPTQ + H-Scale).  The factor's workspace (bytes) and the factor itself; U is
 // also used as scratch for the damped copy of H.
 int64_t gptq_factor_padded(int64_t n);
@@ -120,6 +128,7 @@ cudaError_t read_hessian_device_error(uint32_t* flags);
 cudaError_t read_output_error_device_error(uint32_t* flags);
 cudaError_t read_update_device_error(uint32_t* flags);
 cudaError_t read_gptq_device_error(uint32_t* flags);
+cudaError_t read_hessian_cluster_device_error(uint32_t* flags);
 cudaError_t read_selftest_device_error(uint32_t* flags);
 
 // One CTA waits at most `polls` polls on an mbarrier that nothing arrives on.

@@ -15,6 +15,7 @@
 //                         factor reads the upper triangle only).  K runs in segments of 2048
 //                         tokens, each accumulated from zero and folded into a running sum
 //                         in tensor memory
+//   (hessian_cluster.cu)  the same for widths with few tiles: a cluster per tile splits K
 //   transpose_kernel,     the same for X whose rows are not 16-byte aligned (no TMA): X is
 //   gemm_kernel<1>        transposed into the workspace (tokens contiguous per channel)
 //                         and both operands are K-major
@@ -543,6 +544,10 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
   if (err != cudaSuccess) return err;
   const int64_t tiles_n = (n + kBN - 1) / kBN;
   const int64_t tiles = ((n + kBM - 1) / kBM) * tiles_n;
+  DeviceInfo info;
+  if ((err = current_device_info(&info)) != cudaSuccess) return err;
+  const bool h_aligned = (reinterpret_cast<uintptr_t>(H) & 15) == 0 && ld_h % 4 == 0;
+  const int cluster = hessian_cluster_size(tokens, n, h_aligned, info.sm_count);
   if ((reinterpret_cast<uintptr_t>(x) & 15) == 0 && ld_x % 8 == 0) {
     // X read as it is: 64-channel x 64-token boxes, MN-major operands (kMode 3).  Where n is whole
     // 64-channel groups, X is mapped as [n / 64][tokens][64] and one load takes an operand's two or
@@ -563,6 +568,7 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
     };
     if (encode_x(&map, kBM / 64) != CUDA_SUCCESS || encode_x(&bmap, kBN / 64) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
+    if (cluster > 1) return launch_hessian_cluster(cluster, map, bmap, true, grouped, tokens, n, H, ld_h, stream);
     err = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<3>), (int)kGemmSmemBytes);
     if (err != cudaSuccess) return err;
     gemm_kernel<3><<<(unsigned)tiles, kGemmThreads, kGemmSmemBytes, stream>>>(
@@ -588,6 +594,7 @@ cudaError_t launch_hessian_full(const void* x, int64_t tokens, int64_t n, int64_
       encode(&bmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xt, dims, strides, bbox, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
+  if (cluster > 1) return launch_hessian_cluster(cluster, amap, bmap, false, false, tokens, n, H, ld_h, stream);
   const cudaError_t attr_status =
       ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel<1>), (int)kGemmSmemBytes);
   if (attr_status != cudaSuccess) return attr_status;

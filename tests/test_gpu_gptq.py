@@ -84,6 +84,42 @@ def test_full_hessian_matches_oracle(tokens, n, chunks, view):
     assert hs.hscale_device_error_flags() == 0
 
 
+@pytest.mark.parametrize("tokens,n,view", [
+    (8192, 256, "whole"),            # four segments: clusters of four
+    (8193, 384, "whole"),            # a fifth of one token
+    (18000, 130, "whole"),           # nine segments in clusters of eight; unaligned H rows, K-major operands
+    (10240, 1280, "aligned slice"),  # five segments, clusters of four; widths past one tile
+    (9000, 2000, "whole"),           # clusters of two; n not a multiple of 64
+    (4100, 1001, "whole"),           # two full segments and a third, unaligned rows
+])
+def test_full_hessian_by_clusters(tokens, n, view):
+    """Widths whose tiles are split over a cluster's CTAs: into an H that is not zero, a call adds
+    the sum of its 2048-token segments, bit for bit that of calls of one segment each into a
+    zeroed H; only the tiles on and above the diagonal are written."""
+    x = calib(n, tokens, 300 + n).to(dev())
+    if view == "aligned slice":
+        wide = torch.zeros(tokens, n + 24, dtype=torch.bfloat16, device=dev())
+        wide[:, 8:8 + n] = x
+        x = wide[:, 8:8 + n]
+    H1 = torch.zeros(n, n, dtype=torch.float32, device=dev())
+    H2 = torch.zeros_like(H1)
+    base = torch.full((n, n), 3.0, dtype=torch.float32, device=dev())
+    H3 = base.clone()
+    hs.hscale_hessian_full_accumulate(x, H1)
+    hs.hscale_hessian_full_accumulate(x, H3)
+    for t0 in range(0, tokens, 2048):
+        hs.hscale_hessian_full_accumulate(x[t0:t0 + 2048], H2)
+    torch.cuda.synchronize()
+    i = torch.arange(n, device=dev())
+    written = (i[None, :] // 256 + 1) * 256 > (i[:, None] // 128) * 128
+    assert torch.equal(H1[written], H2[written]) and bool((H1[~written] == 0).all())
+    assert torch.equal(H3[written], (base + H2)[written]) and bool((H3[~written] == 3).all())
+    d = torch.diagonal(H1).double()
+    ref = x.double().square().sum(0)
+    assert bool(((d - ref).abs() <= 1e-5 * ref + 1e-30).all())
+    assert hs.hscale_device_error_flags() == 0
+
+
 def test_full_hessian_one_call_equals_2048_token_calls():
     """The kernel's accumulation segments: one call over 12,000 tokens gives, bit for bit,
     the H of successive calls of 2048 tokens (the last one ragged)."""
