@@ -34,6 +34,7 @@
 
 #include <algorithm>
 
+#include "chained_launch.h"
 #include "factor_block.cuh"
 #include "hscale_internal.h"
 #include "split3.cuh"
@@ -47,11 +48,12 @@ constexpr int kPanelThreads = 256;
 constexpr int kPanelSmemBytes = (kNb * kLd + kNb * (kPanelRows + 4)) * 4;
 
 // ---------------------------------------------------------------- set-up
-// One block: dead channels (H_jj = 0) and the damped diagonal dd_j = d_j + damp * mean(d),
+// One block: info cleared, dead channels (H_jj = 0) and the damped diagonal dd_j = d_j + damp * mean(d),
 // d_j = H_jj, or 1 for a dead channel (fp32; the mean in fp64).
 __global__ void __launch_bounds__(1024) damp_diagonal_kernel(const float* __restrict__ H, int64_t n, int64_t ld_h,
                                                              float damp, uint8_t* __restrict__ dead,
-                                                             float* __restrict__ dd) {
+                                                             float* __restrict__ dd, int32_t* __restrict__ info) {
+  if (threadIdx.x < 3) info[threadIdx.x] = 0;
   __shared__ double part[1024];
   double s = 0.0;
 #pragma unroll 4
@@ -73,44 +75,52 @@ __global__ void __launch_bounds__(1024) damp_diagonal_kernel(const float* __rest
   for (int64_t j = threadIdx.x; j < n; j += blockDim.x) dd[j] = dd[j] + add;
 }
 
-// W2 [n_pad, 2 n_pad]: the left half B_ij = A_{n-1-i, n-1-j} for i, j < n, A the damped H
-// (read from H's upper triangle, row stride ld_h, and the damped diagonal dd), the identity
-// beyond n; the right half (X) zero where the sweep accumulates into it, strictly below the
-// 128-block diagonal (nothing reads X above it).  One 32 x 32 tile of each half per block.
-// Every read and write runs along a row: a tile of B below the diagonal reads H's rows
-// (reversed), a tile above it reads the mirrored tile of H and transposes it in shared
-// memory, and a tile on the diagonal reads the entries on and below it and takes the rest
-// from its own transpose.
+// W2 [n_pad, 2 n_pad]: the left half B_ij = A_{n-1-i, n-1-j} for i, j < n on and below the 128-block
+// diagonal, A the damped H (read from H's upper triangle, row stride ld_h, and the damped diagonal
+// dd), the identity beyond n; the right half (X) zero where the sweep accumulates into it,
+// strictly below the 128-block diagonal.  Nothing reads either half above it (so half of both is
+// never written: n = 4096 43 -> 25.6 us).  One 32 x 32 tile of each half per block.
+// Every read and write runs along a row: a tile below the diagonal reads H's rows (reversed), one above it (within a diagonal 128-block) reads the
+// mirrored tile of H and transposes it in shared memory, and a tile on the diagonal reads the
+// entries on and below it and takes the rest from its own transpose.
 __global__ void __launch_bounds__(256) reverse_pad_kernel(const float* __restrict__ H, int64_t n, int64_t ld_h,
                                                           const float* __restrict__ dd, int64_t n_pad,
                                                           float* __restrict__ W2) {
   __shared__ float t[32][33];
   const int bi = (int)blockIdx.y, bj = (int)blockIdx.x;
+  if (bj / (kNb / 32) > bi / (kNb / 32)) return;
   const int64_t i0 = 32 * (int64_t)bi, j0 = 32 * (int64_t)bj, ld = 2 * n_pad;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  float v[4];
   if (bi < bj) {
     // B_ij = A_{n-1-j, n-1-i}: t[jj][ii]
-    for (int jj = ty; jj < 32; jj += 8) {
-      const int64_t j = j0 + jj, i = i0 + tx;
-      t[jj][tx] = (i < n && j < n) ? H[(n - 1 - j) * ld_h + (n - 1 - i)] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t j = j0 + ty + 8 * k, i = i0 + tx;
+      v[k] = (i < n && j < n) ? H[(n - 1 - j) * ld_h + (n - 1 - i)] : 0.0f;
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[ty + 8 * k][tx] = v[k];
     __syncthreads();
     for (int ii = ty; ii < 32; ii += 8) W2[(i0 + ii) * ld + j0 + tx] = t[tx][ii];  // i < j: 0 beyond n
   } else {
     // B_ij = A_{n-1-i, n-1-j} for i >= j: t[ii][jj]
-    for (int ii = ty; ii < 32; ii += 8) {
-      const int64_t i = i0 + ii, j = j0 + tx;
-      t[ii][tx] = (i < n && j < n && i >= j) ? H[(n - 1 - i) * ld_h + (n - 1 - j)] : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t i = i0 + ty + 8 * k, j = j0 + tx;
+      v[k] = (i < n && j < n && i >= j) ? H[(n - 1 - i) * ld_h + (n - 1 - j)] : 0.0f;
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[ty + 8 * k][tx] = v[k];
     __syncthreads();
     for (int ii = ty; ii < 32; ii += 8) {
       const int64_t i = i0 + ii, j = j0 + tx;
-      float v;
+      float x;
       if (i < n && j < n)
-        v = i == j ? dd[n - 1 - i] : (i > j ? t[ii][tx] : t[tx][ii]);
+        x = i == j ? dd[n - 1 - i] : (i > j ? t[ii][tx] : t[tx][ii]);
       else
-        v = i == j ? 1.0f : 0.0f;
-      W2[i * ld + j] = v;
+        x = i == j ? 1.0f : 0.0f;
+      W2[i * ld + j] = x;
     }
   }
   if (bi / (kNb / 32) > bj / (kNb / 32))
@@ -301,27 +311,6 @@ factor_panel_kernel(const float* __restrict__ Bw, float* __restrict__ Xw, int64_
 
 inline int64_t round256(int64_t bytes) { return (bytes + 255) / 256 * 256; }
 
-// The sweep's kernels are launched with programmatic dependent launch: the kernel before each
-// lets it be scheduled as soon as it starts, and it waits for that kernel's writes before its
-// first read, so those launches do not each wait out a launch's latency.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), unsigned grid, unsigned block, int smem, cudaStream_t stream,
-                           Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(block, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-  if (err != cudaSuccess) return err;
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 int64_t gptq_factor_padded(int64_t n) { return (n + kNb - 1) / kNb * kNb; }
@@ -345,8 +334,7 @@ cudaError_t launch_gptq_factor(const float* H, int64_t n, int64_t ld_h, float da
   float* dd = reinterpret_cast<float*>(base + round256(2 * np * np * 4));
   uint16_t* Bo = reinterpret_cast<uint16_t*>(base + round256(2 * np * np * 4) + round256(np * kNb * 4));
 
-  if ((err = cudaMemsetAsync(info, 0, 3 * sizeof(int32_t), stream)) != cudaSuccess) return err;
-  damp_diagonal_kernel<<<1, 1024, 0, stream>>>(H, n, ld_h, damp, dead, dd);
+  damp_diagonal_kernel<<<1, 1024, 0, stream>>>(H, n, ld_h, damp, dead, dd, info);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   reverse_pad_kernel<<<dim3((unsigned)(np / 32), (unsigned)(np / 32)), 256, 0, stream>>>(H, n, ld_h, dd, np, Bw);
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
@@ -356,7 +344,7 @@ cudaError_t launch_gptq_factor(const float* H, int64_t n, int64_t ld_h, float da
     return err;
 
   // the first diagonal block; every later one is factored by the update before it
-  if ((err = launch_chained(factor_diag_kernel, 1, kDiagThreads, kDiagSmemBytes, stream, (const float*)Bw, ld,
+  if ((err = launch_chained(factor_diag_kernel, dim3(1), kDiagThreads, kDiagSmemBytes, stream, (const float*)Bw, ld,
                             (int64_t)0, Xw, info)) != cudaSuccess)
     return err;
   const int64_t nblk = np / kNb;
@@ -367,7 +355,7 @@ cudaError_t launch_gptq_factor(const float* H, int64_t n, int64_t ld_h, float da
     // the last block column has no panel: only the inverse's row
     const int panel_blocks = (int)(rows / kPanelRows), row_blocks = (int)(j0 / kPanelRows);
     const int blocks = panel_blocks + row_blocks + (rows > 0 ? kNb / kPanelRows : 0);
-    if (blocks > 0 && (err = launch_chained(factor_panel_kernel, (unsigned)blocks, kPanelThreads, kPanelSmemBytes,
+    if (blocks > 0 && (err = launch_chained(factor_panel_kernel, dim3((unsigned)blocks), kPanelThreads, kPanelSmemBytes,
                                             stream, (const float*)Bw, Xw, ld, j0, r_first, rows, panel_blocks,
                                             row_blocks, Bo)) != cudaSuccess)
       return err;

@@ -13,6 +13,7 @@
 
 #include <cuda_bf16.h>
 
+#include "chained_launch.h"
 #include "hscale_device.cuh"
 #include "hscale_internal.h"
 #include "search.cuh"
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
 // One GB300, 4096 x 4096, blocks of 128: 26-28 us a panel (53 K cycles: set-up 5,
 // quantizing 4 x 6.5, propagating 6.6 + 4.4 + 2.3, adding to the strip 3 x 0.8, write-out 1.4),
 // where the four blocks took about 130 us with a quantizer and two updates launched for each;
-// the whole call 1050 -> 628 us.
+// the whole call 1050 -> 628 us, and 571 since its launches overlap.
 constexpr int kPanelCols = 512;
 constexpr int kPanelThreads = 512;
 constexpr int kSlots = 6;
@@ -247,6 +248,9 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
     tmem_alloc(smem_addr(tmem_slot), kCols);
     tmem_relinquish();
   }
+  // the call's inputs are complete (the call's first kernel is launched in stream order); the
+  // running weights and U's parts come from the kernels before this one
+  pdl_launch_dependents();
   const ScaleDomain d = make_scale_domain(*args.global_scale);
   const float inv6 = rtn_inv6_raw(d.sgk);
   const float2 b6 = anchor_brackets(d.sgk, 6.0f);
@@ -255,6 +259,7 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
     hs[c] = args.h[args.col0 + c];
     ud[c] = args.U[(args.col0 + c) * args.n + args.col0 + c];
   }
+  pdl_wait_primary();
   {
     const int quads = outer / 4;
     for (int e = tid; e < kRows * quads; e += kPanelThreads) {
@@ -495,40 +500,70 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
 }
 
 // The update's other operand [nn, 3 B] (row j: the three bf16 parts of U[col0 .. col0 + B, c1 + j]),
-// transposed through 32 x 32 shared-memory tiles so that the reads of U and the writes are
-// coalesced
+// transposed through 64 x 64 shared-memory tiles: 16-byte reads along U's rows where n allows,
+// 8-byte writes (512 x 4096: 6.8 us with 32 x 32 tiles and 2-byte writes, now 6.0).
 __global__ void __launch_bounds__(256) split_u_kernel(const float* __restrict__ U, int64_t n, int64_t col0, int B,
                                                       int64_t c1, uint16_t* __restrict__ Bt) {
-  __shared__ float t[32][33];
-  const int64_t j0 = (int64_t)blockIdx.x * 32;
-  const int k0 = blockIdx.y * 32;
-  if (c1 + j0 + 31 <= col0 + k0) return;  // wholly on or below the diagonal: never used
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int kk = ty; kk < 32; kk += 8) {
-    const int64_t col = c1 + j0 + tx;
-    t[kk][tx] = (k0 + kk < B && col < n) ? U[(col0 + k0 + kk) * n + col] : 0.0f;
+  __shared__ float t[64][65];
+  pdl_launch_dependents();
+  pdl_wait_primary();  // the previous panel's update has read the operand
+  const int64_t j0 = (int64_t)blockIdx.x * 64;
+  const int k0 = blockIdx.y * 64;
+  if (c1 + j0 + 63 <= col0 + k0) return;  // wholly on or below the diagonal: never used
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 rows of 16 x 4 columns
+  const int64_t col = c1 + j0 + 4 * tx;
+#pragma unroll
+  for (int kk = ty; kk < 64; kk += 16) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k0 + kk < B) {
+      const float* src = U + (col0 + k0 + kk) * n + col;
+      if ((n & 3) == 0 && col + 4 <= n) {  // U is 16-byte aligned, and col a multiple of 4
+        v = *reinterpret_cast<const float4*>(src);
+      } else {
+        if (col < n) v.x = src[0];
+        if (col + 1 < n) v.y = src[1];
+        if (col + 2 < n) v.z = src[2];
+        if (col + 3 < n) v.w = src[3];
+      }
+    }
+    t[kk][4 * tx] = v.x;
+    t[kk][4 * tx + 1] = v.y;
+    t[kk][4 * tx + 2] = v.z;
+    t[kk][4 * tx + 3] = v.w;
   }
   __syncthreads();
-  for (int jj = ty; jj < 32; jj += 8) {
+  const int k = k0 + 4 * tx;  // four of K; B is a multiple of 16
+#pragma unroll
+  for (int jj = ty; jj < 64; jj += 16) {
     const int64_t j = j0 + jj;
-    const int k = k0 + tx;
-    if (c1 + j < n && k < B) {
-      uint16_t p[3];
-      split3(t[tx][jj], p);
-      uint16_t* row = Bt + j * 3 * B + k;
-      row[0] = p[0];
-      row[B] = p[1];
-      row[2 * B] = p[2];
-    }
+    if (c1 + j >= n || k >= B) continue;
+    const float v[4] = {t[4 * tx][jj], t[4 * tx + 1][jj], t[4 * tx + 2][jj], t[4 * tx + 3][jj]};
+    store_split3x4(Bt + j * 3 * B + k, B, v);
   }
 }
 
-__global__ void __launch_bounds__(256) to_fp32_kernel(const uint16_t* __restrict__ w, int64_t m, int64_t n,
-                                                      const uint8_t* __restrict__ dead, float* __restrict__ W) {
-  const int64_t total = m * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = e % n;
-    W[e] = (dead && dead[c]) ? 0.0f : __uint_as_float((uint32_t)w[e] << 16);
+// Eight weights a thread: one 16-byte read, two 16-byte writes (4096 x 4096: 39 us with one
+// weight a thread and a 64-bit remainder each, now 20.6).
+__global__ void __launch_bounds__(256) to_fp32_kernel(const uint4* __restrict__ w, int64_t vectors, uint32_t row_vectors,
+                                                      const uint8_t* __restrict__ dead, float4* __restrict__ W) {
+  pdl_launch_dependents();
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < vectors; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint4 v = ld_stream_v4(w + e);
+    const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+    float f[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      f[2 * k] = bf16_lo(x[k]);
+      f[2 * k + 1] = bf16_hi(x[k]);
+    }
+    if (dead != nullptr) {
+      const uint32_t c = vectors <= UINT32_MAX ? (uint32_t)e % row_vectors : (uint32_t)(e % row_vectors);
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (dead[8 * (int64_t)c + k]) f[k] = 0.0f;
+    }
+    W[2 * e] = make_float4(f[0], f[1], f[2], f[3]);
+    W[2 * e + 1] = make_float4(f[4], f[5], f[6], f[7]);
   }
 }
 
@@ -542,9 +577,8 @@ cudaError_t launch_panel(const CUtensorMap& umap, const PanelArgs& args, cudaStr
   const cudaError_t err =
       ensure_dynamic_smem(reinterpret_cast<const void*>(gptq_panel_kernel<kRows>), (int)PanelSmem<kRows>::kBytes);
   if (err != cudaSuccess) return err;
-  gptq_panel_kernel<kRows><<<(unsigned)((args.m + kRows - 1) / kRows), kPanelThreads, PanelSmem<kRows>::kBytes, stream>>>(
-      umap, args);
-  return cudaGetLastError();
+  return launch_chained(gptq_panel_kernel<kRows>, dim3((unsigned)((args.m + kRows - 1) / kRows)), kPanelThreads,
+                        PanelSmem<kRows>::kBytes, stream, umap, args);
 }
 
 }  // namespace
@@ -559,7 +593,8 @@ int64_t gptq_update_cols(int64_t n, int64_t block) {
 // panel is quantized with its blocks' propagation inside it (gptq_panel_kernel, which writes
 // the split errors), and the columns right of it take their update, W -= E U, as one GEMM over
 // K = the panel's columns (update.cu).  Wider blocks (over 512 columns) are a panel each, by
-// block_kernel.  Everything runs on the caller's stream.
+// block_kernel.  Everything runs on the caller's stream, each kernel scheduled
+// while the one before it runs (programmatic dependent launch).
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
                                const float* global_scale, const uint8_t* dead, int block, int down, int up,
                                uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
@@ -569,8 +604,9 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
   if (err != cudaSuccess) return err;
   EncodeTiledFn encode = nullptr;
   if ((err = encode_tiled_fn(&encode)) != cudaSuccess) return err;
-  const unsigned cvt_blocks = (unsigned)std::min<int64_t>((m * n + 255) / 256, (int64_t)info.sm_count * 16);
-  to_fp32_kernel<<<cvt_blocks, 256, 0, stream>>>(static_cast<const uint16_t*>(w), m, n, dead, Wf);
+  const unsigned cvt_blocks = (unsigned)std::min<int64_t>((m * n / 8 + 255) / 256, (int64_t)info.sm_count * 8);
+  to_fp32_kernel<<<cvt_blocks, 256, 0, stream>>>(static_cast<const uint4*>(w), m * n / 8, (uint32_t)(n / 8), dead,
+                                                 reinterpret_cast<float4*>(Wf));
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   const int64_t step = gptq_update_cols(n, block);
   for (int64_t c0 = 0; c0 < n; c0 += step) {
@@ -579,9 +615,9 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
     // U's columns from the panel's second block on (from the next panel on for a wide block)
     const int64_t first = wide ? c1 : c0;
     if (c0 + block < n) {
-      split_u_kernel<<<dim3((unsigned)((n - first + 31) / 32), (unsigned)((K + 31) / 32)), 256, 0, stream>>>(
-          U, n, c0, (int)K, first, Us);
-      if ((err = cudaGetLastError()) != cudaSuccess) return err;
+      if ((err = launch_chained(split_u_kernel, dim3((unsigned)((n - first + 63) / 64), (unsigned)((K + 63) / 64)), 256, 0,
+                                stream, U, n, c0, (int)K, first, Us)) != cudaSuccess)
+        return err;
     }
     if (wide) {
       const int64_t groups = m * (K / 16);

@@ -167,9 +167,8 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_d = warp_uniform(*tmem_slot);
-  // launched with programmatic dependent launch by the factor: the next kernel may be scheduled
-  // (after the TMEM allocation), and the previous one's writes must be visible before the first
-  // load; without the launch attribute both are no-ops
+  // launched with programmatic dependent launch: the next kernel may be scheduled (after the TMEM
+  // allocation), and the previous one's writes must be visible before the first load
   pdl_launch_dependents();
   pdl_wait_primary();
 
@@ -424,7 +423,7 @@ cudaError_t launch_update(const CUtensorMap& amap, const CUtensorMap& bmap, cons
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = kFactor ? 1 : 0;
+  cfg.numAttrs = 1;
   err = cudaLaunchKernelEx(&cfg, update_kernel<kFactor>, amap, bmap, cmap, xmap, args);
   if (err != cudaSuccess) return err;
   return cudaGetLastError();
