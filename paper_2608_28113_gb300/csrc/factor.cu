@@ -20,8 +20,8 @@
 // So the serial part of step j + 1 runs beside the update of step j, and the chain per step is
 // one panel, one tile of the update and one diagonal block.  The first diagonal block has a kernel of its
 // own (factor_diag_kernel).
-// One GB300, n = 4096: 1.05 ms (1.755 ms with the diagonal block, panel, splits and update one
-// after another), of which about 31 steps of 30 us: diagonal block 16, its tile 5, panel 4,
+// One GB300, n = 4096: 0.85 ms (1.755 ms with the diagonal block, panel, splits and update one
+// after another), of which about 31 steps of 25 us: diagonal block 10.5, its tile 5.5, panel 4,
 // launches and hand-over the rest.
 // X = L^-1 is built alongside: row blocks below the diagonal accumulate
 // R_ic = -sum_k L_ik X_kc as the sweep passes, and X_ic = Z_ii R_ic once row block i is reached.
@@ -144,8 +144,7 @@ __global__ void __launch_bounds__(kDiagThreads, 1)
 factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* __restrict__ Xw,
                    int32_t* __restrict__ info) {
   extern __shared__ __align__(16) uint8_t dynamic_smem[];
-  float* S = reinterpret_cast<float*>(dynamic_smem);  // [128][kLd] the block, then L (lower)
-  float* X = S + kNb * kLd;                           // [128][kLd] the inverse (lower)
+  float* S = reinterpret_cast<float*>(dynamic_smem);  // [128][kLd] the block
   const int tid = threadIdx.x;
 
   // programmatic dependent launch on both sides
@@ -158,19 +157,9 @@ factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* 
     const int e = tid + t * kDiagThreads;
     const int r = e >> 5, c = (e & 31) * 4;
     *reinterpret_cast<float4*>(S + r * kLd + c) = *reinterpret_cast<const float4*>(blk + r * ld + c);
-    *reinterpret_cast<float4*>(X + r * kLd + c) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   __syncthreads();
-  factor_block128(0, info, (int32_t)j0);
-  // write-out: Z into Xw's diagonal block (16-byte words).  L_jj itself is not needed again:
-  // the panel uses Z_jj, and the rest of the sweep reads only the blocks below the diagonal.
-  float* xo = Xw + j0 * ld + j0;
-#pragma unroll 4
-  for (int t = 0; t < kNb * kNb / 4 / kDiagThreads; ++t) {
-    const int e = tid + t * kDiagThreads;
-    const int r = e >> 5, c = (e & 31) * 4;
-    *reinterpret_cast<float4*>(xo + r * ld + c) = *reinterpret_cast<const float4*>(X + r * kLd + c);
-  }
+  factor_block128(0, Xw + j0 * ld + j0, ld, info, (int32_t)j0);
 }
 
 // ---------------------------------------------------------------- panel (CUDA cores)

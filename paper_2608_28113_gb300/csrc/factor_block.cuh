@@ -2,7 +2,11 @@
 // inverted by one CTA in shared memory (used by factor.cu for the first block and by the
 // factor's update kernel in update.cu for every later one).
 #pragma once
+#include <cuda_bf16.h>
+
 #include <cstdint>
+
+#include "tma.cuh"
 
 namespace hscale {
 
@@ -10,7 +14,9 @@ constexpr int kNb = 128;                  // block of the sweep
 constexpr int kSub = 16;                  // sub-block of the diagonal factor (one warp)
 constexpr int kLd = kNb + 4;              // padded shared-memory row (16-byte multiple)
 constexpr int kDiagThreads = 512;
-constexpr int kDiagSmemBytes = (2 * kNb * kLd + 4) * 4;
+constexpr int kPlane = kSub + 8;          // row (bf16) of a split operand: eight of them meet no bank twice
+// the block, its current column's splits, two sub-factors' splits, the sub-factor's input
+constexpr int kDiagSmemBytes = kNb * kLd * 4 + 3 * kNb * kPlane * 2 + 2 * 3 * kSub * kPlane * 2 + kSub * kLd * 4;
 
 __device__ __forceinline__ void record_failure(int32_t* info, int32_t order) {
   atomicCAS(reinterpret_cast<int*>(info), 0, order);
@@ -33,9 +39,20 @@ __device__ __forceinline__ float fast_rsqrt(float x) {
   return r;
 }
 
+// The three bf16 parts of a pair of values, packed (x in the low half).
+__device__ __forceinline__ void split3_pair(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+    p[s] = *reinterpret_cast<const uint32_t*>(&v);
+    x = __fsub_rn(x, __uint_as_float(p[s] << 16));
+    y = __fsub_rn(y, __uint_as_float(p[s] & 0xFFFF0000u));
+  }
+}
+
 // One warp factors the 16 x 16 block at A (row stride kLd, lower triangle), A = L L^T, and
-// writes Z = L^-1 (lower, zeros above) at Zo (row stride kLd).  The block's own L is not
-// needed: only Z is written.
+// writes Z = L^-1 (lower, zeros above) as three bf16 parts (split3_pair), transposed, kSub rows of
+// kPlane each, at Zo.  The block's own L is not needed: only Z is written.
 //
 // Two halves of the warp run the same instructions: lane i < 16 holds row i of the block,
 // lane 16 + c holds column c of the unit-lower inverse Y, which starts as the identity.  The
@@ -51,17 +68,19 @@ __device__ __forceinline__ float fast_rsqrt(float x) {
 // 2 x 2 pivot block (1 / d_j+1 = a / det).  Each step forms the next pivot block first, the same
 // in every lane from entries shuffled before the update (no shuffle of updated values on the
 // chain), and the rest of its update fits in the chain's shadow.  The reciprocals are
-// the approximate hardware ones.  A pivot that is not positive is kept in a register (the first
-// one) and recorded once at the end, so no step branches.
+// the approximate hardware ones.  The quick form only notes the ranges of a and det, which a pivot
+// that is not positive leaves too; kFull keeps the first such pivot in a register and records it
+// once at the end, so no step branches.
 //
-// Measured on one GB300: 1.7 K cycles per 16 columns beside the other warps' products; the
+// Measured on one GB300: 1.9 K cycles per 16 columns beside other warps' work; the
 // 32-wide sweep before this one, a Cholesky with square roots on the chain and 64 values per
 // lane, took 7.5 K per 32 columns.
 //
-// Returns whether every pivot was in the range of the quick reciprocals (if not, nothing was
-// recorded and Zo is to be formed again with kFull).
+// Returns whether every pivot was positive and in the range where the quick form's reciprocals and
+// det neither underflow nor overflow (if not, nothing was recorded and Zo is to be formed again
+// with kFull).
 template <bool kFull>
-__device__ __forceinline__ bool factor_sub16(const float* A, float* Zo, int lane, int32_t* info, int32_t base) {
+__device__ __forceinline__ bool factor_sub16(const float* A, uint16_t* Zo, int lane, int32_t* info, int32_t base) {
   const unsigned full = 0xFFFFFFFFu;
   const bool is_row = lane < kSub;
   const int li = lane & (kSub - 1);
@@ -75,11 +94,22 @@ __device__ __forceinline__ bool factor_sub16(const float* A, float* Zo, int lane
     r[k + 3] = is_row ? a.w : (k + 3 == li ? 1.0f : 0.0f);
   }
   int32_t fail = 0;
-  float lo = 1.0f, hi = 1.0f;  // the range of the pivots
-  float ia, ic, r1;
+  float lo = 1.0f, hi = 1.0f, det_lo = 1.0f, det_hi = 1.0f;  // the ranges of a and of det
+  float ia, ic, r1, det;
   // the pivots j and j + 1 from the pivot block [a b; b c] (the same in every lane): ia = 1 / d_j,
   // ic = 1 / d_j+1, r1 = this lane's entry j + 1 after pivot j
   auto pivot = [&](int j, float a, float b, float c) {
+    if (!kFull) {
+      ia = fast_rcp<kFull>(a);
+      det = __fmaf_rn(a, c, -__fmul_rn(b, b));
+      ic = __fmul_rn(a, fast_rcp<kFull>(det));
+      r1 = __fmaf_rn(-__fmul_rn(b, ia), r[j], r[j + 1]);
+      lo = fminf(lo, a);
+      hi = fmaxf(hi, a);
+      det_lo = fminf(det_lo, det);
+      det_hi = fmaxf(det_hi, det);
+      return;
+    }
     const bool bad_a = !(a > 0.0f);
     fail = (fail == 0 && bad_a) ? base + j + 1 : fail;
     a = bad_a ? 1.0f : a;
@@ -87,16 +117,12 @@ __device__ __forceinline__ bool factor_sub16(const float* A, float* Zo, int lane
     const float m = __fmul_rn(b, ia);
     // det 2^-e, e the exponent of a, so that it has the magnitude of d_j+1 = det / a
     const float as = __uint_as_float((__float_as_uint(a) & 0x007FFFFFu) | 0x3F800000u);  // a 2^-e
-    const float bs = __fmul_rn(b, __uint_as_float(0x7F000000u - (__float_as_uint(a) & 0x7F800000u)));
-    float det = __fmaf_rn(as, c, -__fmul_rn(bs, b));
-    if (kFull) det = __fmul_rn(as, __fmaf_rn(-m, b, c));
+    det = __fmul_rn(as, __fmaf_rn(-m, b, c));
     const bool bad_c = !(det > 0.0f);
     fail = (fail == 0 && bad_c) ? base + j + 2 : fail;
     det = bad_c ? as : det;
     ic = __fmul_rn(as, fast_rcp<kFull>(det));
     r1 = __fmaf_rn(-m, r[j], r[j + 1]);
-    lo = fminf(lo, fminf(a, det));
-    hi = fmaxf(hi, fmaxf(a, det));
   };
   pivot(0, __shfl_sync(full, r[0], 0), __shfl_sync(full, r[0], 1), __shfl_sync(full, r[1], 1));
 #pragma unroll
@@ -125,235 +151,250 @@ __device__ __forceinline__ bool factor_sub16(const float* A, float* Zo, int lane
     zs[j] = __fmul_rn(ja, fast_rsqrt<kFull>(ja));
     zs[j + 1] = __fmul_rn(jc, fast_rsqrt<kFull>(jc));
   }
-  if (!kFull && !(lo >= 0x1p-100f && hi <= 0x1p100f)) return false;
+  // a NaN passes the minima and maxima, but reaches every later pivot
+  if (!kFull && !(lo >= 0x1p-50f && hi <= 0x1p50f && det_lo >= 0x1p-100f && det_hi <= 0x1p100f && det > 0.0f))
+    return false;
   if (fail != 0 && lane == 0) record_failure(info, fail);
-  // lane 16 + c holds column c of Y: row i is zero above the diagonal (i < c)
-  if (!is_row) {
+  // lane 16 + c holds column c of Y (row i is zero above the diagonal, i < c) and writes its rows
+  // 0-7 of Z, lane c the rows 8-15
+  float z[kSub / 2];
 #pragma unroll
-    for (int i = 0; i < kSub; ++i) Zo[i * kLd + li] = i >= li ? __fmul_rn(r[i], zs[i]) : 0.0f;
+  for (int i = 0; i < kSub / 2; ++i) {
+    const float lower = __shfl_sync(full, r[i + 8], li + kSub);
+    const float y = is_row ? __fmul_rn(lower, zs[i + 8]) : __fmul_rn(r[i], zs[i]);
+    z[i] = i + (is_row ? 8 : 0) >= li ? y : 0.0f;
   }
+  uint32_t part[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint32_t pr[3];
+    split3_pair(z[2 * i], z[2 * i + 1], pr);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) part[s][i] = pr[s];
+  }
+#pragma unroll
+  for (int s = 0; s < 3; ++s)
+    *reinterpret_cast<uint4*>(Zo + (s * kSub + li) * kPlane + (is_row ? 8 : 0)) =
+        make_uint4(part[s][0], part[s][1], part[s][2], part[s][3]);
   __syncwarp();
   return true;
 }
-static __device__ __noinline__ void factor_sub16_full(const float* A, float* Zo, int lane, int32_t* info, int32_t base) {
+static __device__ __noinline__ void factor_sub16_full(const float* A, uint16_t* Zo, int lane, int32_t* info,
+                                                      int32_t base) {
   factor_sub16<true>(A, Zo, lane, info, base);
 }
 
-__device__ __forceinline__ void block_factor(const float* A, float* Zo, int lane, int32_t* info, int32_t base) {
-  if (!factor_sub16<false>(A, Zo, lane, info, base)) factor_sub16_full(A, Zo, lane, info, base);
+// ---------------------------------------------------------------- warp-level products
+// mma.sync m16n8k16 on bf16 parts, fp32 accumulation.  These products are too small and too
+// dependent on each other for the tcgen05 units (one 16 x 16 x 16 product at a time, needed by the
+// next one); they run on registers.  A 16 x 16 block is a fragment of two n8 halves:
+// f[h][0..1] row g, columns 8 h + 2 t, + 1; f[h][2..3] row g + 8 (g = lane / 4, t = lane % 4).
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// One warp's product of 16 x 16 blocks in shared memory (row stride kLd = 4 mod 32 words).
-// A lane holds rows h, h + 8 and four columns: 4 cl + q (kNT false) or cl + 4 q (kNT true).
-// Per four m, A's rows are 16-byte words, and B is read either row by row (kNT false: B[m][c]
-// at B + m kLd + c) or in place from the transposed operand's rows (kNT true: B[m][c] at
-// B + c kLd + m), 16-byte words too.  Shared-memory reads bound these products (a 16-byte read
-// takes four cycles of the SM, two when neighbouring lanes i and i ^ 1, or i and i ^ 2, share
-// the address; measured), so h leaves out lane bit 0, cl lane bit 1, and the rows and columns
-// are dealt so that no read or write meets a bank twice.
-//   acc[r][q] += sum_m A[h + 8 r][m] B[m][column q]   (-= with kNeg), over m in order
-__device__ __forceinline__ int block_row(int lane) { return ((lane >> 3) & 3) + 2 * (lane & 2); }
-__device__ __forceinline__ int block_col(int lane) { return ((lane >> 1) & 2) + (lane & 1); }
-
-template <bool kNT, bool kNeg>
-__device__ __forceinline__ void block_mma(float (&acc)[2][4], const float* A, const float* B, int lane) {
-  const int h = block_row(lane), cl = block_col(lane);
+// A block as the A operand of three parts (the accumulator's layout is the operand's).
+__device__ __forceinline__ void split_fragment(const float (&f)[2][4], uint32_t (&a)[3][4]) {
 #pragma unroll
-  for (int m = 0; m < kSub; m += 4) {
-    float b[4][4];  // b[m][q]
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 v = kNT ? *reinterpret_cast<const float4*>(B + (cl + 4 * q) * kLd + m)
-                           : *reinterpret_cast<const float4*>(B + (m + q) * kLd + 4 * cl);
-      const float e[4] = {v.x, v.y, v.z, v.w};
+    for (int q = 0; q < 2; ++q) {
+      uint32_t p[3];
+      split3_pair(f[h][2 * q], f[h][2 * q + 1], p);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) (kNT ? b[k][q] : b[q][k]) = kNeg ? -e[k] : e[k];
+      for (int s = 0; s < 3; ++s) a[s][2 * h + q] = p[s];
     }
+}
+// f = A B^T to fp32 accuracy, A and B 16 x 16 in three parts each: the six products above 2^-24, the
+// small ones in a sum of their own, which also halves the chain of dependent MMAs.
+// b[s][0..1]: rows 0-7 of B's part s (columns 0-7, 8-15), b[s][2..3]: rows 8-15.
+__device__ __forceinline__ void block_product(float (&f)[2][4], const uint32_t (&a)[3][4], const uint32_t (&b)[3][4]) {
+  float e[2][4];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const float4 v = *reinterpret_cast<const float4*>(A + (h + 8 * r) * kLd + m);
-      const float a[4] = {v.x, v.y, v.z, v.w};
+  for (int h = 0; h < 2; ++h)
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
+    for (int q = 0; q < 4; ++q) e[h][q] = f[h][q] = 0.0f;
+  auto both = [&](float (&d)[2][4], int i, int j) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] = __fmaf_rn(a[k], b[k][q], acc[r][q]);
-    }
+    for (int h = 0; h < 2; ++h) mma16816(d[h], a[i], b[j][2 * h], b[j][2 * h + 1]);
+  };
+  both(e, 0, 2);
+  both(f, 0, 1);
+  both(e, 2, 0);
+  both(f, 1, 0);
+  both(e, 1, 1);
+  both(f, 0, 0);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f[h][q] = __fadd_rn(f[h][q], e[h][q]);
+}
+// The block B of that product (kTransposed: stored as its transpose) from shared memory: three
+// parts of kPlane-wide rows, `part` elements apart.
+template <bool kTransposed>
+__device__ __forceinline__ void load_block(uint32_t (&b)[3][4], const uint16_t* B, int part, int lane) {
+  // the 8 x 8 block of lanes 8 i .. 8 i + 7: rows 8 (i / 2) of B, columns 8 (i % 2)
+  const int n = (lane >> 1) & 8, k = lane & 8;
+  const uint32_t at = smem_addr(B + ((kTransposed ? k : n) + (lane & 7)) * kPlane + (kTransposed ? n : k));
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const uint32_t src = at + (uint32_t)(s * part * 2);
+    if (kTransposed)
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(b[s][0]), "=r"(b[s][1]), "=r"(b[s][2]), "=r"(b[s][3])
+                   : "r"(src)
+                   : "memory");
+    else
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(b[s][0]), "=r"(b[s][1]), "=r"(b[s][2]), "=r"(b[s][3])
+                   : "r"(src)
+                   : "memory");
   }
 }
-__device__ __forceinline__ void block_zero(float (&acc)[2][4]) {
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[0][q] = acc[1][q] = 0.0f;
-}
-template <bool kNT>
-__device__ __forceinline__ void block_load(float (&acc)[2][4], const float* T, int lane) {
-  const int h = block_row(lane), cl = block_col(lane);
-#pragma unroll
-  for (int r = 0; r < 2; ++r)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[r][q] = T[(h + 8 * r) * kLd + (kNT ? cl + 4 * q : 4 * cl + q)];
-}
-template <bool kNT>
-__device__ __forceinline__ void block_store(const float (&acc)[2][4], float* T, int lane) {
-  const int h = block_row(lane), cl = block_col(lane);
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    if (kNT) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) T[(h + 8 * r) * kLd + cl + 4 * q] = acc[r][q];
-    } else {
-      *reinterpret_cast<float4*>(T + (h + 8 * r) * kLd + 4 * cl) =
-          make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-    }
-  }
-}
 
-// P = P Z^T in place
-__device__ __forceinline__ void block_panel(float* P, const float* Z, int lane) {
-  float acc[2][4];
-  block_zero(acc);
-  block_mma<true, false>(acc, P, Z, lane);
-  __syncwarp();
-  block_store<true>(acc, P, lane);
-}
-// T = Z T in place
-__device__ __forceinline__ void block_row_solve(float* T, const float* Z, int lane) {
-  float acc[2][4];
-  block_zero(acc);
-  block_mma<false, false>(acc, Z, T, lane);
-  __syncwarp();
-  block_store<false>(acc, T, lane);
-}
-// T = -sum over count blocks of L (16 columns further each) times X (16 rows further each)
-__device__ __forceinline__ void block_row_sum(float* T, const float* L, const float* X, int count, int lane) {
-  float acc[2][4];
-  block_zero(acc);
-  for (int k = 0; k < count; ++k) block_mma<false, true>(acc, L + k * kSub, X + k * kSub * kLd, lane);
-  block_store<false>(acc, T, lane);
-}
-// C -= A B^T
-__device__ __forceinline__ void block_sub_nt(float* C, const float* A, const float* B, int lane) {
-  float acc[2][4];
-  block_load<true>(acc, C, lane);
-  block_mma<true, true>(acc, A, B, lane);
-  block_store<true>(acc, C, lane);
-}
-// The same for a 16 x 32 tile, C -= A B^T: a lane holds rows 2 h, 2 h + 1, 2 h + 8,
-// 2 h + 9 and columns cl + 8 q (q < 4), which reads 32 bytes of shared memory per 16 products instead of 48.
-__device__ __forceinline__ void wide_sub_nt(float* C, const float* A, const float* B, int lane) {
-  const int h2 = (lane & 2) + ((lane >> 2) & 4), cl = (lane & 1) + ((lane >> 1) & 2) + ((lane >> 1) & 4);
-  constexpr int kRow[4] = {0, 1, 8, 9};
-  float acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[r][q] = C[(h2 + kRow[r]) * kLd + cl + 8 * q];
-#pragma unroll
-  for (int m = 0; m < kSub; m += 4) {
-    float4 b[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) b[q] = *reinterpret_cast<const float4*>(B + (cl + 8 * q) * kLd + m);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float4 a = *reinterpret_cast<const float4*>(A + (h2 + kRow[r]) * kLd + m);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        acc[r][q] = __fmaf_rn(-a.x, b[q].x, acc[r][q]);
-        acc[r][q] = __fmaf_rn(-a.y, b[q].y, acc[r][q]);
-        acc[r][q] = __fmaf_rn(-a.z, b[q].z, acc[r][q]);
-        acc[r][q] = __fmaf_rn(-a.w, b[q].w, acc[r][q]);
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) C[(h2 + kRow[r]) * kLd + cl + 8 * q] = acc[r][q];
-}
-
-// Factor the 128 x 128 block in S (row stride kLd, lower triangle; B_jj = L_jj L_jj^T) and
-// invert the factor: Z_jj = L_jj^-1 in X (zero on entry above the diagonal; lower).  The block
-// is an 8 x 8 grid of 16 x 16 blocks, taken in columns p = 0..7:
-//   (a) warp 0 factors and inverts the block on the diagonal (factor_sub16): Z_p into X_pp;
-//   (b) one warp each: the blocks below it, L_ip = B_ip Z_p^T (i > p, in place), and the
-//       inverse's row, X_pc = Z_p T_pc (c < p, in place);
-//   (c) right-looking in S, B_ik -= L_ip L_kp^T (p < k <= i), and left-looking in X, the next
-//       row's T_p+1,c = -sum_{k=c..p} L_p+1,k X_kc (c <= p).
-// Warp 0 runs ahead: of (b) and (c) it takes only the products on the way to the next diagonal
-// block, L_p+1,p and B_p+1,p+1, and goes on to its (a) while the other warps run the rest,
-// taking the products of (c) one at a time from a counter (the longest sums first).  A column
-// costs the slower of the two.  Left-looking in X keeps (c) even: 19 to 28 products in every
-// column, where right-looking would put 34 in the first and 7 in the last.
-// Bound by the reads of shared memory in (c) (16 bytes a lane take two to four cycles of the SM)
-// and, behind them, by the sub-factors.  One GB300: about 30 K cycles per 128-block, against 52 K
-// for 32-wide tiles without look-ahead (the whole factor at n = 4096: 1755 -> 1540 us from this).
+// Factor the 128 x 128 block B in shared memory (at byte `offset` of the kernel's dynamic shared
+// memory, row stride kLd; its lower triangle) and write the factor's inverse, Z = L^-1, to xo (row
+// stride ld, zeros above the diagonal).
 //
-// S, X and the counter of (c) sit at byte `offset` of the kernel's dynamic shared memory
-// (kDiagSmemBytes): the function finds them there itself, so that its accesses are shared-memory
-// instructions (through a pointer whose origin the compiler does not see they are generic ones:
-// 21.7 us a block instead of 16).
+// Elimination of the tall matrix [B ; I], taken in 16-wide columns p = 0..7: with
+// Z_p = L_pp^-1 (factor_sub16), every row block has P = V_p Z_p^T (for a row block of B that
+// is L_rp; for row block c of I, X_pc^T, a block of the inverse) and V_i -= P L_ip^T for the columns
+// i > p.  So a row block needs from the others only Z_p and the L_ip: each of the 16 warps
+// holds one row block in registers for the whole elimination (eight 16 x 16 blocks), warps 0-7
+// those of B, 8-15 those of I; the products are warp-level MMAs on three bf16 parts, and only
+// Z_p and the column's L_ip go through shared memory, as parts.
+//
+// What bounds it is the chain of the sub-factors, about 1.9 K of a column's 2.7 K cycles.  The warp of
+// row block p + 1 carries it: with Z_p it forms P and from that its diagonal block, both in
+// registers (P's fragment is either operand of P P^T), and factors it, while the other warps
+// update their columns.  Row block r of B is done with column r - 1, so the lead passes from warp
+// to warp, each of which has split its first block before Z_p comes.  The warp index has to be
+// uniform: with one taken per thread the n = 4096 factor took 934 us in place of 868.
+//
+// One GB300: 10.5 us a block inside the update kernel, against 16.4 with the products on CUDA cores
+// through shared memory, whose reads bound them (n = 4096 factor 1030 -> 852 us).
 constexpr int kGrid16 = kNb / kSub;
-static __device__ __noinline__ void factor_block128(uint32_t offset, int32_t* info, int32_t j0) {
+static __device__ __noinline__ void factor_block128(uint32_t offset, float* __restrict__ xo, int64_t ld, int32_t* info,
+                                                    int32_t j0) {
   extern __shared__ __align__(16) uint8_t dynamic_smem[];
-  float* S = reinterpret_cast<float*>(dynamic_smem + offset);
-  float* X = S + kNb * kLd;
-  int* next = reinterpret_cast<int*>(X + kNb * kLd);
-  const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // column -1 is only warp 0's first sub-factor
+  const float* S = reinterpret_cast<const float*>(dynamic_smem + offset);
+  uint16_t* Lp = reinterpret_cast<uint16_t*>(dynamic_smem + offset + kNb * kLd * 4);
+  uint16_t* Zp = Lp + 3 * kNb * kPlane;  // two of them
+  float* D = reinterpret_cast<float*>(Zp + 2 * 3 * kSub * kPlane);
+  const int lane = (int)threadIdx.x & 31, warp = (int)warp_uniform(threadIdx.x >> 5);
+  const int g = lane >> 2, t = lane & 3, r = warp & 7;
+  const bool of_b = warp < kGrid16;
+  float v[kGrid16][2][4];  // the row block's columns p, p + 1, ...
+  if (warp != 0) {
+#pragma unroll
+    for (int i = 0; i < kGrid16; ++i)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 8 * h + 2 * t;
+        float2 x = make_float2(0.0f, 0.0f), y = x;
+        if (of_b && i <= r) {
+          x = *reinterpret_cast<const float2*>(S + (kSub * r + g) * kLd + kSub * i + c);
+          y = *reinterpret_cast<const float2*>(S + (kSub * r + g + 8) * kLd + kSub * i + c);
+        }
+        v[i][h][0] = x.x; v[i][h][1] = x.y; v[i][h][2] = y.x; v[i][h][3] = y.y;
+      }
+  }
+
 #pragma unroll 1
-  for (int p = -1; p < kGrid16; ++p) {
-    const int c0 = p * kSub, d0 = c0 + kSub;
-    const float* Zp = X + c0 * kLd + c0;
-    if (warp == 0) {
-      if (p + 1 == kGrid16) break;
-      float* D = S + d0 * kLd + d0;
-      if (p >= 0) {
-        block_panel(S + d0 * kLd + c0, Zp, lane);
-        __syncwarp();
-        asm volatile("bar.arrive 1, 512;" ::: "memory");  // L_p+1,p is in place
-        block_sub_nt(D, S + d0 * kLd + c0, S + d0 * kLd + c0, lane);
-        __syncwarp();
-      }
-      block_factor(D, X + d0 * kLd + d0, lane, info, j0 + d0);
-    } else if (p >= 0) {
-      // (b): c < p on warps 1..p, i > p + 1 on warps p + 1..6
-      if (warp <= p) {
-        block_row_solve(X + c0 * kLd + (warp - 1) * kSub, Zp, lane);
-      } else if (warp + 1 < kGrid16) {
-        block_panel(S + (warp + 1) * kSub * kLd + c0, Zp, lane);
-      } else if (tid == kDiagThreads - 1) {
-        *next = 0;
-      }
-      if (p + 1 == kGrid16) break;
-      asm volatile("bar.sync 1, 512;" ::: "memory");
-      // (c): T_p+1,c for c = 0..p, then rows i > p + 1 of S, two blocks (i, k), (i, k + 1)
-      // at a time
-      for (;;) {
-        int e = 0;
-        if (lane == 0) e = atomicAdd(next, 1);
-        e = __shfl_sync(0xFFFFFFFFu, e, 0);
-        if (e <= p) {
-          block_row_sum(X + d0 * kLd + e * kSub, S + d0 * kLd + e * kSub, X + e * kSub * kLd + e * kSub, p + 1 - e,
-                        lane);
-          continue;
-        }
-        int i = p + 2, k = e - (p + 1);  // row i has (i - p + 1) / 2 tiles
-        while (i < kGrid16 && k >= (i - p + 1) / 2) {
-          k -= (i - p + 1) / 2;
-          ++i;
-        }
-        if (i >= kGrid16) break;
-        k = p + 1 + 2 * k;
-        float* C = S + i * kSub * kLd + k * kSub;
-        const float* L = S + i * kSub * kLd + c0;
-        if (k < i)
-          wide_sub_nt(C, L, S + k * kSub * kLd + c0, lane);
-        else
-          block_sub_nt(C, L, L, lane);
+  for (int p = 0; p < kGrid16; ++p) {
+    if (warp == p) {  // this row block of B has only its sub-factor left
+      const float* A = p == 0 ? S : D;
+      uint16_t* Zn = Zp + (p & 1) * 3 * kSub * kPlane;
+      const int32_t base = j0 + kSub * p;
+      if (!factor_sub16<false>(A, Zn, lane, info, base)) factor_sub16_full(A, Zn, lane, info, base);
+      // the row block's registers are the sub-factor's until here
+#pragma unroll
+      for (int i = 0; i < kGrid16; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[i][h][q] = 0.0f;
+    }
+    uint32_t a[3][4];
+    if (!of_b && r == p) {  // its first column
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[0][h][q] = g + 8 * (q >> 1) == 8 * h + 2 * t + (q & 1) ? 1.0f : 0.0f;
+    }
+    const bool active = of_b ? r > p : r <= p;
+    const bool lead = of_b && r == p + 1;
+    if (active) split_fragment(v[0], a);
+    __syncthreads();  // Z_p is in place, the reads of the last column's L are done
+    // the lead first: the others' products would share its tensor cores
+    if (!lead && p + 1 < kGrid16) asm volatile("bar.sync 1, 512;" ::: "memory");
+    float P[2][4] = {};
+    if (active) {
+      uint32_t z[3][4];
+      load_block<true>(z, Zp + (p & 1) * 3 * kSub * kPlane, kSub * kPlane, lane);
+      block_product(P, a, z);
+      split_fragment(P, a);
+      if (of_b) {
+#pragma unroll
+        for (int s = 0; s < 3; ++s)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+              *reinterpret_cast<uint32_t*>(Lp + (s * kNb + kSub * r + g + 8 * q) * kPlane + 8 * h + 2 * t) =
+                  a[s][2 * h + q];
       }
     }
-    __syncthreads();
+    if (!of_b) {
+      // X[16 p + column][16 r + row]; zeros above the block diagonal (p < r)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          xo[(int64_t)(kSub * p + 8 * h + 2 * t + (q & 1)) * ld + kSub * r + g + 8 * (q >> 1)] = P[h][q];
+    }
+    if (p + 1 == kGrid16) break;
+    if (lead) {
+      uint32_t b[3][4];
+      float d[2][4];
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        b[s][0] = a[s][0];
+        b[s][1] = a[s][2];
+        b[s][2] = a[s][1];
+        b[s][3] = a[s][3];
+      }
+      block_product(d, a, b);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          *reinterpret_cast<float2*>(D + (g + 8 * q) * kLd + 8 * h + 2 * t) = make_float2(
+              __fsub_rn(v[1][h][2 * q], d[h][2 * q]), __fsub_rn(v[1][h][2 * q + 1], d[h][2 * q + 1]));
+      __syncwarp();
+      asm volatile("bar.arrive 1, 512;" ::: "memory");  // L_p+1,p is in place
+    } else {
+      asm volatile("bar.sync 2, 480;" ::: "memory");  // the column's L is in place
+      if (active) {
+        const int last = of_b ? r - p : kGrid16 - 1 - p;
+#pragma unroll
+        for (int k = 1; k < kGrid16; ++k)
+          if (k <= last) {
+            uint32_t b[3][4];
+            float f[2][4];
+            load_block<false>(b, Lp + kSub * (p + k) * kPlane, kNb * kPlane, lane);
+            block_product(f, a, b);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) v[k - 1][h][q] = __fsub_rn(v[k][h][q], f[h][q]);
+          }
+      }
+    }
   }
-  __syncthreads();
 }
 
 }  // namespace hscale

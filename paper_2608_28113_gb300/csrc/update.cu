@@ -334,33 +334,19 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
       // the reduce-adds complete before the CTA ends
       if (lane == 0) bulk_wait_all();
     }
-  } else if (diagonal) {
-    // warps past the epilogue: the inverse's block starts as zero, in the ring once the MMAs have
-    // read it
-    if (mbar_wait(&acc_full[0], 0u)) {
-      float* X = reinterpret_cast<float*>(smem) + kNb * kLd;
-      for (int e = (int)threadIdx.x - (2 + kEpiWarps) * 32; e < kNb * kLd / 4; e += kDiagThreads - (2 + kEpiWarps) * 32)
-        reinterpret_cast<float4*>(X)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    } else {
-      atomicOr(failed, 1u);
-    }
   }
   tc_fence_before_sync();
   __syncthreads();
   const bool bad = *failed != 0;
   if (bad && threadIdx.x == 0) atomicOr(&g_update_flags, kErrMbarTimeout);
   if (kFactor && diagonal) {
-    const float* X = reinterpret_cast<const float*>(smem) + kNb * kLd;
-    if (!bad) factor_block128(offset, args.info, args.order0);
     // Z_j+1 into the diagonal block of the inverse (zeros above its diagonal)
     float* xo = args.X + args.order0;
-#pragma unroll 4
-    for (int t = 0; t < kNb * kNb / 4 / kDiagThreads; ++t) {
-      const int e = (int)threadIdx.x + t * kDiagThreads;
-      const int r = e >> 5, c = (e & 31) * 4;
-      const float nan = __int_as_float(0x7FC00000);
-      *reinterpret_cast<float4*>(xo + r * args.ld + c) =
-          bad ? make_float4(nan, nan, nan, nan) : *reinterpret_cast<const float4*>(X + r * kLd + c);
+    if (!bad) {
+      factor_block128(offset, xo, args.ld, args.info, args.order0);
+    } else {
+      for (int e = (int)threadIdx.x; e < kNb * kNb; e += kDiagThreads)
+        xo[(e / kNb) * args.ld + e % kNb] = __int_as_float(0x7FC00000);
     }
   } else if (bad && warp >= 2 && warp < 2 + kEpiWarps) {
     // a wait that ran out makes the CTA's tiles NaN

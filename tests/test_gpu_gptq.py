@@ -206,6 +206,20 @@ def test_factor_reports_a_matrix_that_is_not_positive_definite():
     assert 1 <= info[0] <= n and info[1] == 0 and info[2] == 0
 
 
+@pytest.mark.parametrize("order", [1, 2, 15, 16, 17, 33, 128, 129, 250])
+def test_factor_names_the_failed_pivot(order):
+    """Near the identity (off-diagonal sums below 0.5, so every other pivot stays positive) with one
+    entry at -5: the failed pivot is that entry, wherever it lies in its 2 x 2, 16 x 16 and 128 x 128
+    block, and the sweep still ends with finite values."""
+    n = 250
+    noise = np.random.default_rng(order).uniform(-1e-3, 1e-3, (n, n))
+    H = np.eye(n) + noise + noise.T
+    H[n - order, n - order] = -5.0
+    U, dead, info = gpu_factor(H.astype(np.float32))
+    assert list(info) == [order, 0, 0]
+    assert np.isfinite(U).all()
+
+
 def gpu_gptq(w, U32, h32, s_g, block, down, up, dead=None):
     m, n = w.shape
     codes = torch.empty(m, n // 16, dtype=torch.uint8, device=dev())
