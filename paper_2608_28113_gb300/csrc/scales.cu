@@ -357,14 +357,17 @@ __device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_
 // W, the codes and the nibbles are 2-D views: row r starts at element r * ld_w of w, byte
 // r * ld_i of the initial codes, byte r * ld_c of the codes and 8-byte word r * ld_p of the
 // nibbles.
+// The warp index is uniform for the compiler here and in the schedules below, so a unit's row, column
+// and branches are kept once per warp (28672 x 8192, global scale included: 521 -> 504 us; 3001 x 3216
+// with the 4over6 start 39.1 -> 38.0).
 template <bool kFourOverSix>
 __global__ void __launch_bounds__(kRefineThreads, 7)
 refine_kernel(const uint4* __restrict__ w, int64_t ld_w, const float* __restrict__ h, int64_t m, int ng,
               const float* __restrict__ global_scale, const uint8_t* init_codes, int64_t ld_i,
               int down, int up, uint8_t* codes_out, int64_t ld_c, uint2* __restrict__ packed_out, int64_t ld_p) {
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5);
+  const int64_t warp_global = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   const int64_t warps_total = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int chunks = (ng + 31) / 32;
   const int64_t units = m * chunks;
@@ -580,8 +583,8 @@ refine_linear_kernel(const uint4* __restrict__ w, const float* __restrict__ h, i
                      const float* __restrict__ global_scale, const uint8_t* init_codes, int down, int up,
                      uint8_t* codes_out, uint2* __restrict__ packed_out) {
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5);
+  const int64_t warp_global = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   const int64_t warps_total = ((int64_t)gridDim.x * blockDim.x) >> 5;
 
   __shared__ float4 tab[128];
@@ -660,8 +663,8 @@ refine_shared_kernel(const uint4* __restrict__ w, const float* __restrict__ h, u
                      const uint8_t* init_codes, int down, int up, uint8_t* codes_out,
                      uint2* __restrict__ packed_out, unsigned* __restrict__ next) {
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const uint32_t warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5);
+  const uint32_t warp_global = blockIdx.x * (blockDim.x >> 5) + (uint32_t)warp;
   const uint32_t warps_total = (gridDim.x * blockDim.x) >> 5;
 
   __shared__ float4 tab[128];
@@ -757,7 +760,7 @@ refine_sm_kernel(const uint4* __restrict__ w, const float* __restrict__ h, uint3
                  const uint8_t* init_codes, int down, int up, uint8_t* codes_out,
                  uint2* __restrict__ packed_out) {
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5);
   __shared__ float4 tab[128];
   __shared__ __align__(16) uint4 stage[kSmWarps][2][64];
   __shared__ unsigned next_unit;
@@ -840,7 +843,7 @@ refine_flat_kernel(const uint4* __restrict__ w, int64_t row_words, const float* 
                    uint32_t ng, const float* __restrict__ global_scale, const uint8_t* init_codes, int64_t ld_i,
                    int down, int up, uint8_t* codes_out, int64_t ld_c, uint2* __restrict__ packed_out, int64_t ld_p) {
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
+  const int warp = (int)warp_uniform(threadIdx.x >> 5);
   __shared__ float4 tab[128];
   __shared__ __align__(16) uint4 stage[kSmWarps][2][64];
   __shared__ unsigned next_unit;
