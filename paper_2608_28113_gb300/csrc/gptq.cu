@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
 // One GB300, 4096 x 4096, blocks of 128: 26-28 us a panel (53 K cycles: set-up 5,
 // quantizing 4 x 6.5, propagating 6.6 + 4.4 + 2.3, adding to the strip 3 x 0.8, write-out 1.4),
 // where the four blocks took about 130 us with a quantizer and two updates launched for each;
-// the whole call 1050 -> 628 us, and 571 since its launches overlap.
+// the whole call 1050 -> 628 us, 567 since its launches overlap, 554 with update.cu's last tiles
+// halved.
 constexpr int kPanelCols = 512;
 constexpr int kPanelThreads = 512;
 constexpr int kSlots = 6;

@@ -71,6 +71,7 @@ struct UpdateArgs {
   int K;            // columns of A and B
   int rows, cols;   // of C; kFactor: the trailing square's size (twice)
   int tiles;
+  int whole;        // tiles from here on are 128 columns wide, two to a 128 x 256 tile (!kFactor)
   // kFactor
   int xcols;        // columns of the inverse
   float* C;         // [rows, cols] (kFactor: the trailing square)
@@ -80,13 +81,13 @@ struct UpdateArgs {
   int32_t* info;
 };
 
-// The tiles of one CTA in turn: position (tm, tn), columns, and whether the tile belongs to the
-// inverse (kFactor).
+// The tiles of one CTA in turn: rows from 128 tm, columns [col0, col_end), and whether the tile
+// belongs to the inverse (kFactor).
 template <bool kFactor>
 struct Tiles {
   const UpdateArgs& s;
   int t, step, tiles_n, first;
-  int tm, tn;
+  int tm, col0, col_end;
   bool inverse;
   __device__ explicit Tiles(const UpdateArgs& args) : s(args), first(0), tm(0) {
     tiles_n = ((kFactor ? s.xcols : s.cols) + kBN - 1) / kBN;
@@ -111,17 +112,19 @@ struct Tiles {
       }
       const int k = t - first;
       inverse = k > tm / 2;
-      tn = inverse ? k - (tm / 2 + 1) : k;
+      col0 = (inverse ? k - (tm / 2 + 1) : k) * kBN;
+      col_end = inverse ? s.xcols : (tm + 1) * kBM;
     } else {
-      tm = t / tiles_n;
-      tn = t - tm * tiles_n;
+      const bool half = t >= s.whole;
+      const int tile = half ? s.whole + (t - s.whole) / 2 : t;
+      tm = tile / tiles_n;
+      col0 = (tile - tm * tiles_n) * kBN + (half ? ((t - s.whole) & 1) * (kBN / 2) : 0);
+      col_end = half ? min(s.cols, col0 + kBN / 2) : s.cols;
       inverse = false;
     }
   }
-  // columns of the tile that are wanted; the first row of B
-  __device__ int col_end() const { return kFactor ? (inverse ? s.xcols : (tm + 1) * kBM) : s.cols; }
-  __device__ bool narrow() const { return col_end() - tn * kBN <= 128; }
-  __device__ int b_row() const { return (kFactor && inverse ? s.rows : 0) + tn * kBN; }
+  __device__ bool narrow() const { return col_end - col0 <= 128; }
+  __device__ int b_row() const { return (kFactor && inverse ? s.rows : 0) + col0; }
 };
 
 // The parts of product p, the small products first.
@@ -178,8 +181,8 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     uint32_t s = 0, parity = 1;  // position in the ring, over all of the CTA's tiles
     bool go = true;
     for (Tiles<kFactor> T(args); go && T.valid(); T.next()) {
-      // kFactor: A and B are one array, whose 128-row boxes amap has
-      const bool narrow = kFactor && T.narrow();
+      // B's boxes of 128 rows: amap's in kFactor, where A and B are one array, otherwise xmap's
+      const bool narrow = T.narrow();
       const int a_row = T.tm * kBM, b_row = T.b_row();
       for (int p = 0; p < kProducts && go; ++p) {
         for (int c = 0; c < chunks; ++c) {
@@ -191,7 +194,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
             uint8_t* st = smem + s * kStageBytes;
             mbar_arrive_expect_tx(&full[s], narrow ? 2 * kHalfTileBytes : kStageBytes);
             tma_load_3d(st, &amap, c * kBK, part_a(p), a_row, &full[s], policy);
-            tma_load_3d(st + kHalfTileBytes, narrow ? &amap : &bmap, c * kBK, part_b(p), b_row, &full[s], policy);
+            tma_load_3d(st + kHalfTileBytes, narrow ? (kFactor ? &amap : &xmap) : &bmap, c * kBK, part_b(p), b_row, &full[s], policy);
           }
           __syncwarp();
           if (++s == kStages) {
@@ -280,7 +283,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
       for (Tiles<kFactor> T(args); T.valid(); T.next(), ++i) {
         const uint32_t a = i & 1u;
         const CUtensorMap* map = kFactor && T.inverse ? &xmap : &cmap;
-        const int row0 = T.tm * kBM + (int)quarter * 32, col0 = T.tn * kBN + (int)half * 128, col_end = T.col_end();
+        const int row0 = T.tm * kBM + (int)quarter * 32, col0 = T.col0 + (int)half * 128, col_end = T.col_end;
         // subtract 32 columns of the tile (values p) from C
         auto subtract = [&](const uint32_t (&p)[32], int c) {
           // the previous box must have been read out of the buffer
@@ -352,9 +355,9 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     // a wait that ran out makes the CTA's tiles NaN
     for (Tiles<kFactor> T(args); T.valid(); T.next()) {
       float* base = kFactor && T.inverse ? args.X : args.C;
-      const int row = T.tm * kBM + (warp & 3) * 32 + lane, c0 = T.tn * kBN + ((warp - 2) >> 2) * 128;
+      const int row = T.tm * kBM + (warp & 3) * 32 + lane, c0 = T.col0 + ((warp - 2) >> 2) * 128;
       if (row < args.rows)
-        for (int c = c0; c < min(c0 + 128, T.col_end()); ++c)
+        for (int c = c0; c < min(c0 + 128, T.col_end); ++c)
           base[(int64_t)row * args.ld + c] = __int_as_float(0x7FC00000);
     }
   }
@@ -422,20 +425,29 @@ cudaError_t launch_split_update(const void* a, const void* b, int64_t rows, int6
   EncodeTiledFn encode = nullptr;
   cudaError_t err = encode_tiled_fn(&encode);
   if (err != cudaSuccess) return err;
-  CUtensorMap amap, bmap, cmap;
+  CUtensorMap amap, bmap, bhalf, cmap;
   if ((err = encode_operand(encode, &amap, a, rows, K, kBM)) != cudaSuccess) return err;
   if ((err = encode_operand(encode, &bmap, b, cols, K, kBN)) != cudaSuccess) return err;
+  if ((err = encode_operand(encode, &bhalf, b, cols, K, kBN / 2)) != cudaSuccess) return err;
   if ((err = encode_target(encode, &cmap, C, rows, cols, ld)) != cudaSuccess) return err;
   const int64_t tiles = ((rows + kBM - 1) / kBM) * ((cols + kBN - 1) / kBN);
-  if (tiles > INT32_MAX) return cudaErrorInvalidValue;
+  if (tiles > INT32_MAX / 2) return cudaErrorInvalidValue;
   UpdateArgs args = {};
   args.K = (int)K;
   args.rows = (int)rows;
   args.cols = (int)cols;
-  args.tiles = (int)tiles;
+  // The tiles of a last round that leaves half of the SMs idle are halved: the round is bound by each
+  // SM's MMAs and loads.  Above that line some SM would have two halves, a whole tile's time.  4096 x
+  // 4096 in blocks of 128: three of its seven updates, 567 -> 554 us; quarters where three quarters are
+  // idle gave no more.
+  DeviceInfo info;
+  if ((err = current_device_info(&info)) != cudaSuccess) return err;
+  const int last = (int)(tiles % info.sm_count);
+  args.whole = 2 * last <= info.sm_count ? (int)tiles - last : (int)tiles;
+  args.tiles = (int)tiles + ((int)tiles - args.whole);
   args.C = C;
   args.ld = ld;
-  return launch_update<false>(amap, bmap, cmap, cmap, args, stream);
+  return launch_update<false>(amap, bmap, cmap, bhalf, args, stream);
 }
 
 cudaError_t launch_factor_update(const void* operand, int64_t rows, int64_t xcols, float* C, float* X, int64_t ld,

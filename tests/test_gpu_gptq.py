@@ -308,6 +308,22 @@ def test_gptq_panel_shapes(m, n, block):
     assert hs.hscale_device_error_flags() == 0
 
 
+@pytest.mark.parametrize("m,n", [(1300, 4096), (300, 4224), (2500, 1920)])
+def test_gptq_rows_do_not_depend_on_the_others(m, n):
+    """The update's last round of tiles may be halved, by how many there are, so by m; every
+    element's products are summed in one order all the same: a call on some of the rows gives the
+    bytes of the call on all of them."""
+    w = wl.weight(m, n, 0.02, 31)
+    x = torch.randn(2 * n, n, device=dev(), generator=torch.Generator(device=dev()).manual_seed(7))
+    H32 = (x.T @ x / (2 * n)).cpu().numpy()
+    U, dead, _ = gpu_factor(H32)
+    U32, h32, s_g = U.astype(np.float32), np.ascontiguousarray(np.diag(H32)), 4e-5
+    codes, packed = gpu_gptq(w, U32, h32, s_g, 128, 4, 4)
+    for r0, r1 in ((0, 128), (m // 2 - 57, m // 2 + 40), (m - 200, m)):
+        c, p = gpu_gptq(w[r0:r1].contiguous(), U32, h32, s_g, 128, 4, 4)
+        assert np.array_equal(c, codes[r0:r1]) and np.array_equal(p, packed[r0:r1])
+
+
 def test_gptq_zero_groups_keep_the_initial_code():
     """Groups that are all zero (dead channels) score zero under every code: the tie rule keeps
     the initial code, 1, and the nibbles are zero."""
