@@ -20,8 +20,8 @@
 // So the serial part of step j + 1 runs beside the update of step j, and the chain per step is
 // one panel, one tile of the update and one diagonal block.  The first diagonal block has a kernel of its
 // own (factor_diag_kernel).
-// One GB300, n = 4096: 0.85 ms (1.755 ms with the diagonal block, panel, splits and update one
-// after another), of which about 31 steps of 25 us: diagonal block 10.5, its tile 5.5, panel 4,
+// One GB300, n = 4096: 0.80 ms in a graph (1.755 ms with the diagonal block, panel, splits and update one
+// after another), of which about 31 steps of 23 us: diagonal block 11, its tile 4, panel 4,
 // launches and hand-over the rest.
 // X = L^-1 is built alongside: row blocks below the diagonal accumulate
 // R_ic = -sum_k L_ik X_kc as the sweep passes, and X_ic = Z_ii R_ic once row block i is reached.

@@ -25,7 +25,11 @@
 //   * CTA 0 takes only the next diagonal block: its update goes from tensor memory to shared
 //     memory, where the CTA factors and inverts it (factor_block128) and writes the inverse
 //     Z_j+1, while the other CTAs run the rest of the update.  So the serial diagonal block
-//     runs beside the update and not after it.
+//     runs beside the update and not after it.  It is the step's critical path, so nothing of it
+//     goes through the ring: the operand (A and B are the same rows) is loaded once, whole, and the
+//     block by TMA too.  One GB300: 4.0 us to the tile in shared memory, of which the MMAs take 2.0,
+//     against 5.5 through the ring with the block's rows read by the epilogue's threads (n = 4096
+//     factor 847 -> 802 us in a graph).
 //
 // One GB300: the K = 512 update of 4096 x 3584 takes 56 us with the operands' first touch from
 // HBM (the tensor pipe 73 % busy); what it cannot hide are the ends of the last round of tiles
@@ -50,8 +54,11 @@ constexpr uint32_t kBoxBytes = kBoxCols * kBoxRows * 4;
 // the ring, barriers in a 1 KB block (keeping the boxes 1 KB aligned for the 128-byte swizzle),
 // the epilogue's boxes
 constexpr uint32_t kUpdateSmemBytes = 1024 /* alignment */ + kStages * kStageBytes + 1024 + kEpiWarps * kBoxBytes;
+constexpr uint32_t kDiagOperandBytes = 6 * kHalfTileBytes;  // the next diagonal block's
 constexpr int kLoopThreads = 320;  // TMA warp, MMA warp, 8 epilogue warps
 static_assert(kDiagSmemBytes <= (int)(kStages * kStageBytes), "the diagonal block is factored in the ring");
+static_assert(kDiagOperandBytes + kNb * kNb * 4 <= kStages * kStageBytes, "its operands and itself are loaded into the ring");
+static_assert(kNb * kLd * 4 <= (int)kDiagOperandBytes, "it takes the operands' place");
 
 __device__ uint32_t g_update_flags = 0;
 
@@ -180,7 +187,21 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(policy));
     uint32_t s = 0, parity = 1;  // position in the ring, over all of the CTA's tiles
     bool go = true;
-    for (Tiles<kFactor> T(args); go && T.valid(); T.next()) {
+    if (diagonal) {
+      if (elect_one()) {
+        // A and B are the same rows: three parts of two K steps, then the block itself in the
+        // reduce-add's boxes
+        mbar_arrive_expect_tx(&full[0], kDiagOperandBytes);
+        for (int e = 0; e < 6; ++e)
+          tma_load_3d(smem + e * kHalfTileBytes, &amap, (e & 1) * kBK, e >> 1, 0, &full[0], policy);
+        mbar_arrive_expect_tx(&full[1], kNb * kNb * 4);
+        for (int e = 0; e < 16; ++e)
+          tma_load_2d(smem + kDiagOperandBytes + e * kBoxBytes, &cmap, (e & 3) * (int)kBoxCols,
+                      (e >> 2) * (int)kBoxRows, &full[1], policy);
+      }
+      __syncwarp();
+    }
+    for (Tiles<kFactor> T(args); !diagonal && go && T.valid(); T.next()) {
       // B's boxes of 128 rows: amap's in kFactor, where A and B are one array, otherwise xmap's
       const bool narrow = T.narrow();
       const int a_row = T.tm * kBM, b_row = T.b_row();
@@ -209,7 +230,20 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
   } else if (warp == 1) {
     uint32_t s = 0, parity = 0, i = 0;  // i counts the CTA's tiles
     bool ok = true;
-    for (Tiles<kFactor> T(args); ok && T.valid(); T.next(), ++i) {
+    if (diagonal) {
+      ok = mbar_wait_warp(&full[0], 0u);
+      tc_fence_after_sync();
+      if (ok && elect_one()) {
+        for (int p = 0; p < kProducts; ++p)
+          for (int c = 0; c < 2; ++c)
+            umma_bf16_block(tmem_d, smem_desc_k_sw128(smem_addr(smem + (2 * part_a(p) + c) * kHalfTileBytes)),
+                            smem_desc_k_sw128(smem_addr(smem + (2 * part_b(p) + c) * kHalfTileBytes)),
+                            idesc_bf16_f32(kBM, kNb), kBK / 16, (uint32_t)(p > 0 || c > 0));
+        umma_commit(smem_addr(&acc_full[0]));
+      }
+      __syncwarp();
+    }
+    for (Tiles<kFactor> T(args); !diagonal && ok && T.valid(); T.next(), ++i) {
       const uint32_t idesc = T.narrow() ? idesc_bf16_f32(kBM, 128) : idesc_bf16_f32(kBM, kBN);
       const uint32_t a = i & 1u, d = tmem_d + a * kBN;
       // the accumulator's previous tile (two back) must have been read out of TMEM
@@ -250,29 +284,25 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     const uint32_t lane_base = (quarter * 32u) << 16;
     uint8_t* box = smem + kStages * kStageBytes + 1024 + (uint32_t)(warp - 2) * kBoxBytes;
     if (diagonal) {
-      // the next diagonal block: this thread's row, 64 columns, in place of the tile
+      // the next diagonal block: this thread's row, 64 columns, less the tile
       const int row = (int)quarter * 32 + lane;
-      const float* src = args.C + (int64_t)row * args.ld + 64 * half;
-      float b[64];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float4 v = reinterpret_cast<const float4*>(src)[k];
-        b[4 * k] = v.x; b[4 * k + 1] = v.y; b[4 * k + 2] = v.z; b[4 * k + 3] = v.w;
-      }
-      if (mbar_wait(&acc_full[0], 0u)) {
+      if (mbar_wait(&full[1], 0u) && mbar_wait(&acc_full[0], 0u)) {
         tc_fence_after_sync();
-        float* S = reinterpret_cast<float*>(smem) + row * kLd + 64 * half;
+        float* S = reinterpret_cast<float*>(smem) + row * kLd + 64 * half;  // over the operands
 #pragma unroll
         for (int c = 0; c < 64; c += 32) {
+          const uint8_t* src = smem + kDiagOperandBytes + (4 * quarter + 2 * half + c / 32) * kBoxBytes + lane * 128;
           uint32_t p[32];
           tmem_ld_32x32b_x32(tmem_d + lane_base + 64 * half + (uint32_t)c, p);
           tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 32; k += 4)
+          for (int k = 0; k < 32; k += 4) {
+            // the 128-byte swizzle holds 16-byte chunk i of a row at i ^ (row & 7)
+            const float4 b = *reinterpret_cast<const float4*>(src + ((k / 4) ^ (lane & 7)) * 16);
             *reinterpret_cast<float4*>(S + c + k) =
-                make_float4(__fsub_rn(b[c + k], __uint_as_float(p[k])), __fsub_rn(b[c + k + 1], __uint_as_float(p[k + 1])),
-                            __fsub_rn(b[c + k + 2], __uint_as_float(p[k + 2])),
-                            __fsub_rn(b[c + k + 3], __uint_as_float(p[k + 3])));
+                make_float4(__fsub_rn(b.x, __uint_as_float(p[k])), __fsub_rn(b.y, __uint_as_float(p[k + 1])),
+                            __fsub_rn(b.z, __uint_as_float(p[k + 2])), __fsub_rn(b.w, __uint_as_float(p[k + 3])));
+          }
         }
       } else {
         atomicOr(failed, 1u);
