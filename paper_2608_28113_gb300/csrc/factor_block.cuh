@@ -275,7 +275,9 @@ __device__ __forceinline__ void load_block(uint32_t (&b)[3][4], const uint16_t* 
 // uniform: with one taken per thread the n = 4096 factor took 934 us in place of 868.
 //
 // One GB300: 10.5 us a block inside the update kernel, against 16.4 with the products on CUDA cores
-// through shared memory, whose reads bound them (n = 4096 factor 1030 -> 852 us).
+// through shared memory, whose reads bound them (n = 4096 factor 1030 -> 852 us in a graph); about
+// 0.3 us less since the others no longer wait for the lead's L_p+1,p before their own P (837 -> 825
+// eager).
 constexpr int kGrid16 = kNb / kSub;
 static __device__ __noinline__ void factor_block128(uint32_t offset, float* __restrict__ xo, int64_t ld, int32_t* info,
                                                     int32_t j0) {
@@ -308,6 +310,7 @@ static __device__ __noinline__ void factor_block128(uint32_t offset, float* __re
     if (warp == p) {  // this row block of B has only its sub-factor left
       const float* A = p == 0 ? S : D;
       uint16_t* Zn = Zp + (p & 1) * 3 * kSub * kPlane;
+      __syncwarp();  // D is in place
       const int32_t base = j0 + kSub * p;
       if (!factor_sub16<false>(A, Zn, lane, info, base)) factor_sub16_full(A, Zn, lane, info, base);
       // the row block's registers are the sub-factor's until here
@@ -329,8 +332,6 @@ static __device__ __noinline__ void factor_block128(uint32_t offset, float* __re
     const bool lead = of_b && r == p + 1;
     if (active) split_fragment(v[0], a);
     __syncthreads();  // Z_p is in place, the reads of the last column's L are done
-    // the lead first: the others' products would share its tensor cores
-    if (!lead && p + 1 < kGrid16) asm volatile("bar.sync 1, 512;" ::: "memory");
     float P[2][4] = {};
     if (active) {
       uint32_t z[3][4];
@@ -358,6 +359,7 @@ static __device__ __noinline__ void factor_block128(uint32_t offset, float* __re
     }
     if (p + 1 == kGrid16) break;
     if (lead) {
+      asm volatile("bar.arrive 1, 512;" ::: "memory");  // L_p+1,p is in place
       uint32_t b[3][4];
       float d[2][4];
 #pragma unroll
@@ -374,10 +376,8 @@ static __device__ __noinline__ void factor_block128(uint32_t offset, float* __re
         for (int q = 0; q < 2; ++q)
           *reinterpret_cast<float2*>(D + (g + 8 * q) * kLd + 8 * h + 2 * t) = make_float2(
               __fsub_rn(v[1][h][2 * q], d[h][2 * q]), __fsub_rn(v[1][h][2 * q + 1], d[h][2 * q + 1]));
-      __syncwarp();
-      asm volatile("bar.arrive 1, 512;" ::: "memory");  // L_p+1,p is in place
     } else {
-      asm volatile("bar.sync 2, 480;" ::: "memory");  // the column's L is in place
+      asm volatile("bar.sync 1, 512;" ::: "memory");  // the column's L is in place
       if (active) {
         const int last = of_b ? r - p : kGrid16 - 1 - p;
 #pragma unroll
