@@ -243,6 +243,10 @@ __device__ __forceinline__ uint32_t nonzero_nibbles(uint32_t x) {
   return x & 0x11111111u;
 }
 
+// kFromGroup: the exact decisions select the weight from the group's registers and do not read it
+// back, which is quicker in pack_kernel and slower in the search kernels (28672 x 8192 in a graph
+// 489.6 -> 491.3 us).
+template <bool kFromGroup = false>
 __device__ __forceinline__ uint2 quantize_pack(const Group& G, uint32_t c, float inv, float sgk, float pw,
                                                const uint16_t* wg) {
   const float ilo = __fmul_rn(inv, kBracketLo), ihi = __fmul_rn(inv, kBracketHi);
@@ -263,7 +267,14 @@ __device__ __forceinline__ uint2 quantize_pack(const Group& G, uint32_t c, float
         const int sh = __ffs(flagged) - 1;  // 4 * (element index within the word)
         flagged &= flagged - 1;
         const uint32_t nib = (lo[wd] >> sh) & 0xFu;  // the lower magnitude code, with the sign
-        const float a = __fmul_rn(__uint_as_float(((uint32_t)wg[8 * wd + (sh >> 2)] & 0x7FFFu) << 16), pw);
+        float a;  // the element's magnitude
+        if (kFromGroup) {
+          const float2 p0 = sh & 16 ? G.a[4 * wd + 2] : G.a[4 * wd], p1 = sh & 16 ? G.a[4 * wd + 3] : G.a[4 * wd + 1];
+          const float2 p = sh & 8 ? p1 : p0;
+          a = fabsf(sh & 4 ? p.y : p.x);
+        } else {
+          a = __fmul_rn(__uint_as_float(((uint32_t)wg[8 * wd + (sh >> 2)] & 0x7FFFu) << 16), pw);
+        }
         const uint32_t k = e2m1_code_between(a, nib & 7u, l, sgk);
         lo[wd] = (lo[wd] & ~(0xFu << sh)) | (((nib & 8u) | k) << sh);
       }
@@ -911,7 +922,9 @@ refine_flat_kernel(const uint4* __restrict__ w, int64_t row_words, const float* 
 }
 
 // ---------------------------------------------------------------- pack with given codes
-// Two groups in flight per thread, the reciprocals from a table (14336 x 4096: 37.7 -> 33.2 us).  Bound
+// Two groups in flight per thread, the reciprocals from a table (14336 x 4096: 37.7 -> 33.2 us), and
+// the rare exact decisions on the registers' values and not on a second read (with the passes before
+// it 77.7 -> 75.6; every second warp has such a group where the global scale is short).  Bound
 // by the loads' latency at 52 registers a thread (32 warps an SM); 40 registers spill and are slower.
 template <bool kWide>
 __global__ void __launch_bounds__(256) pack_kernel(const uint4* __restrict__ w, int64_t groups,
@@ -940,7 +953,7 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint4* __restrict__ w, 
       Group G;
       unpack_group(a[u], b[u], d.pw, G);
       const uint32_t cu = c[u] < 1 ? 1u : (c[u] > kE4M3MaxCode ? kE4M3MaxCode : c[u]);
-      packed_out[gu] = quantize_pack(G, cu, inv[cu], d.sgk, d.pw,
+      packed_out[gu] = quantize_pack<true>(G, cu, inv[cu], d.sgk, d.pw,
                                      reinterpret_cast<const uint16_t*>(w) + gu * 16);
     }
   }
