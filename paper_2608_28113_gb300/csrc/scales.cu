@@ -53,6 +53,7 @@
 #include <algorithm>
 #include <atomic>
 
+#include "chained_launch.h"
 #include "hscale_device.cuh"
 #include "hscale_internal.h"
 #include "search.cuh"
@@ -94,8 +95,18 @@ __device__ __forceinline__ uint32_t block_amax(const uint4* __restrict__ w, int6
 }
 
 // Each block's amax into its own 16-bit slot of parts (so nothing has to be cleared first), or,
-// with parts = nullptr, all of them into *amax_bits (which must be 0).
+// with parts = nullptr, all of them into *amax_bits (which must be 0 once the kernel before this one
+// has finished).
 constexpr int kAmaxParts = 128;  // 16-bit slots in the 256-byte workspace
+// From kAmaxSharedElems weights on the blocks share one word and are of 256 threads, so that they
+// find room on SMs that a search or a Hessian pass keeps busy; one of 1024 waits for half an SM to be
+// free at once.  One GB300: the 70B MLP block's step, whose three scale passes run beside both, 1.860
+// ms with 128 blocks of 1024 threads at every size, 1.827 with this rule, the decoder layer's 1.207 and
+// 1.192; alone, 14336 x 4096 with codes and packing 76.1 and 69.0 us, 28672 x 8192 and 4096 x 4096 with
+// their searches the same, 3001 x 3216 37.6 us with the slots and 39.7 with the shared word, whose
+// clearing is a launch more.
+constexpr int64_t kAmaxSharedElems = 1 << 24;
+constexpr int kAmaxSharedThreads = 256, kAmaxSharedBlocks = 512;
 __global__ void __launch_bounds__(kAmaxThreads) amax_kernel(const uint4* __restrict__ w, int64_t nvec,
                                                             uint32_t* __restrict__ amax_bits,
                                                             uint16_t* __restrict__ parts) {
@@ -104,11 +115,19 @@ __global__ void __launch_bounds__(kAmaxThreads) amax_kernel(const uint4* __restr
   const uint32_t m = block_amax(w, nvec, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
                                 (int64_t)gridDim.x * blockDim.x, warp_max);
   if (threadIdx.x == 0) {
+    pdl_wait_primary();  // clear_kernel, when launched behind it; otherwise a no-op
     if (parts != nullptr)
       parts[blockIdx.x] = (uint16_t)m;
     else if (m)
       atomicMax(amax_bits, m);
   }
+}
+
+// *word = 0 for the amax_kernel behind it, which reads W meanwhile: this launch waits for all work
+// before it, so W is complete when that kernel starts.
+__global__ void __launch_bounds__(32) clear_kernel(uint32_t* word) {
+  pdl_launch_dependents();
+  if (threadIdx.x == 0) *word = 0;
 }
 
 __device__ __forceinline__ float global_scale_of(uint32_t amax_bits) {
@@ -1015,6 +1034,11 @@ namespace {
 
 inline bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
 
+// The blocks of amax_kernel that share one word.
+unsigned amax_shared_blocks(int64_t nvec) {
+  return (unsigned)std::min<int64_t>((nvec + kAmaxSharedThreads - 1) / kAmaxSharedThreads, kAmaxSharedBlocks);
+}
+
 // The kernel's grid for `items` units of work, `per_thread` of them per thread and step.
 template <auto kKernel>
 unsigned stream_grid(int64_t items, int threads, int per_thread, int sm_count) {
@@ -1033,7 +1057,7 @@ cudaError_t launch_rtn(const void* w, int64_t groups, const uint32_t* amax, int 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = nparts ? 1 : 0;  // behind amax_kernel of the same call only
+  cfg.numAttrs = w ? 1 : 0;  // behind amax_kernel of the same call only
   const cudaError_t err = cudaLaunchKernelEx(&cfg, rtn_codes_kernel<kWide>, static_cast<const uint4*>(w), groups, amax,
                                              nparts, global_scale, codes);
   return err != cudaSuccess ? err : cudaGetLastError();
@@ -1042,11 +1066,8 @@ cudaError_t launch_rtn(const void* w, int64_t groups, const uint32_t* amax, int 
 }  // namespace
 
 cudaError_t launch_amax(const void* w, int64_t count, uint32_t* amax_bits, cudaStream_t stream) {
-  DeviceInfo info;
-  cudaError_t err = current_device_info(&info);
-  if (err != cudaSuccess) return err;
-  const unsigned blocks = stream_grid<amax_kernel>(count / 8, kAmaxThreads, 1, info.sm_count);
-  amax_kernel<<<blocks, kAmaxThreads, 0, stream>>>(static_cast<const uint4*>(w), count / 8, amax_bits, nullptr);
+  amax_kernel<<<amax_shared_blocks(count / 8), kAmaxSharedThreads, 0, stream>>>(static_cast<const uint4*>(w), count / 8,
+                                                                              amax_bits, nullptr);
   return cudaGetLastError();
 }
 
@@ -1064,14 +1085,22 @@ cudaError_t launch_rtn_scales(const void* w, int64_t m, int64_t n, void* workspa
     small_scale_kernel<<<kSmallScaleCluster, kAmaxThreads, 0, stream>>>(static_cast<const uint4*>(w), nvec, global_scale);
     return cudaGetLastError();
   }
-  // an even number of slots: the reader takes two a word (a block without a share writes 0)
-  const int parts =
-      ((int)std::min<int64_t>({(nvec + kAmaxThreads - 1) / kAmaxThreads, (int64_t)kAmaxParts, (int64_t)info.sm_count}) + 1) &
-      ~1;
-  amax_kernel<<<(unsigned)parts, kAmaxThreads, 0, stream>>>(static_cast<const uint4*>(w), nvec, nullptr,
-                                                           static_cast<uint16_t*>(workspace));
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  const uint32_t* words = static_cast<const uint32_t*>(workspace);
+  uint32_t* words = static_cast<uint32_t*>(workspace);
+  int parts = 0;
+  if (m * n >= kAmaxSharedElems) {
+    clear_kernel<<<1, 32, 0, stream>>>(words);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    err = launch_chained(amax_kernel, dim3(amax_shared_blocks(nvec)), kAmaxSharedThreads, 0, stream,
+                         static_cast<const uint4*>(w), nvec, words, nullptr);
+  } else {
+    // an even number of slots: the reader takes two a word (a block without a share writes 0)
+    parts = ((int)std::min<int64_t>({(nvec + kAmaxThreads - 1) / kAmaxThreads, (int64_t)kAmaxParts,
+                                     (int64_t)info.sm_count}) + 1) & ~1;
+    amax_kernel<<<(unsigned)parts, kAmaxThreads, 0, stream>>>(static_cast<const uint4*>(w), nvec, nullptr,
+                                                             static_cast<uint16_t*>(workspace));
+    err = cudaGetLastError();
+  }
+  if (err != cudaSuccess) return err;
   return aligned32(w) ? launch_rtn<true>(w, m * (n / 16), words, parts, global_scale, codes, info.sm_count, stream)
                       : launch_rtn<false>(w, m * (n / 16), words, parts, global_scale, codes, info.sm_count, stream);
 }

@@ -244,6 +244,31 @@ def test_streaming_passes_over_sizes_and_alignments(m, n, shift):
     assert np.all(np.abs(dw[:, :n] + dw[:, n_pad:n_pad + n] - ref) <= 2.0 ** -17 * np.abs(ref) + 1e-45)
 
 
+@pytest.mark.parametrize("m,n", [(4095, 4096), (4096, 4096), (1025, 16384), (4111, 4112)])
+def test_global_scale_where_its_blocks_begin_to_share_one_word(m, n):
+    """Sizes on both sides of 2^24 weights: the maximum at either end of the matrix counts, a later call
+    with a smaller one gives the smaller scale whatever the workspace held, and the sharded entry
+    point's word agrees.  A maximum of bf16 weights is exact, so the scale is amax / 2688 rounded once."""
+    w = torch.full((m, n), 2.0 ** -10, dtype=torch.bfloat16, device=dev())
+    flat = w.view(-1)
+    ws = torch.full((hs.hscale_rtn_workspace_bytes(),), 0xFF, dtype=torch.uint8, device=dev())
+    sg = torch.zeros(1, dtype=torch.float32, device=dev())
+    word = torch.zeros(1, dtype=torch.int32, device=dev())
+    codes = torch.empty(m, n // 16, dtype=torch.uint8, device=dev())
+    for at, v in ((m * n - 1, -1.5), (0, 1.25), (m * n // 2 + 3, 0.75), (m * n - 8, 0.5), (None, 2.0 ** -10)):
+        if at is not None:
+            flat[at] = v
+        for out in (None, codes):
+            sg.fill_(-1.0)
+            hs.hscale_rtn_scales(w, sg, out, ws)
+            assert sg.item() == float(np.float32(abs(v)) / np.float32(2688.0))
+        hs.hscale_amax_bits(w, word)
+        assert word.item() == int(np.float32(abs(v)).view(np.uint32)) >> 16
+        if at is not None:
+            assert codes.view(-1)[at // 16].item() == 126  # the group of the maximum: 448
+            flat[at] = 2.0 ** -10
+
+
 def exact_tie_matrix():
     """Groups whose max sits exactly on each E4M3 ladder value and midpoint, under
     s_g = 2^-10 (amax = 2688 * 2^-10): RTN ties are decided by round-half-even."""
