@@ -141,8 +141,7 @@ __global__ void __launch_bounds__(256) reverse_out_kernel(const float* __restric
 // The diagonal block at (j0, j0) of Bw: Z_jj into Xw's diagonal block (zeros above the
 // diagonal).  One CTA.  Only the lower triangle of the block is used.
 __global__ void __launch_bounds__(kDiagThreads, 1)
-factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* __restrict__ Xw,
-                   int32_t* __restrict__ info) {
+factor_diag_kernel(const float* Bw, int64_t ld, int64_t j0, float* Xw, int32_t* info) {
   extern __shared__ __align__(16) uint8_t dynamic_smem[];
   float* S = reinterpret_cast<float*>(dynamic_smem);  // [128][kLd] the block
   const int tid = threadIdx.x;
@@ -182,8 +181,8 @@ factor_diag_kernel(const float* __restrict__ Bw, int64_t ld, int64_t j0, float* 
 // One GB300, n = 4096: this one kernel takes the place of two (products, then splits), whose
 // launches took 8.2 and 6.1 us a step.
 __global__ void __launch_bounds__(kPanelThreads)
-factor_panel_kernel(const float* __restrict__ Bw, float* __restrict__ Xw, int64_t ld, int64_t j0, int64_t r_first,
-                    int64_t rows, int panel_blocks, int row_blocks, uint16_t* __restrict__ Bo) {
+factor_panel_kernel(const float* Bw, float* Xw, int64_t ld, int64_t j0, int64_t r_first, int64_t rows, int panel_blocks,
+                    int row_blocks, uint16_t* Bo) {
   extern __shared__ __align__(16) uint8_t dynamic_smem[];
   float* sm = reinterpret_cast<float*>(dynamic_smem);
   constexpr int kRl = kPanelRows + 4;

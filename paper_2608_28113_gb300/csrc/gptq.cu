@@ -186,7 +186,7 @@ __device__ __forceinline__ void tmem_ld_rows(uint32_t src, uint32_t (&r)[32]) { 
 __device__ __forceinline__ void tmem_ld_rows(uint32_t src, uint32_t (&r)[16]) { tmem_ld_32x32b_x16(src, r); }
 
 struct PanelArgs {
-  const float* W;  // running weights [m, n]
+  const float* W;  // running weights [m, n], written by the kernels before this one
   const float* h;
   const float* U;
   const float* global_scale;
@@ -504,7 +504,7 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
 // transposed through 64 x 64 shared-memory tiles: 16-byte reads along U's rows where n allows,
 // 8-byte writes (512 x 4096: 6.8 us with 32 x 32 tiles and 2-byte writes, now 6.0).
 __global__ void __launch_bounds__(256) split_u_kernel(const float* __restrict__ U, int64_t n, int64_t col0, int B,
-                                                      int64_t c1, uint16_t* __restrict__ Bt) {
+                                                      int64_t c1, uint16_t* Bt) {
   __shared__ float t[64][65];
   pdl_launch_dependents();
   pdl_wait_primary();  // the previous panel's update has read the operand

@@ -117,7 +117,7 @@ __device__ __forceinline__ bool spin_or_fail(uint64_t* bar, uint32_t parity, con
 template <int CS>
 __global__ void __launch_bounds__(kThreads, 3)
 hessian_colsumsq_kernel(const __grid_constant__ CUtensorMap xmap, int64_t row0, int64_t rows,
-                        int n, float* __restrict__ h, int64_t rows_per_cta, int x_ready) {
+                        int n, float* h, int64_t rows_per_cta, int x_ready) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full_bar[kStages];

@@ -108,8 +108,7 @@ constexpr int kAmaxParts = 128;  // 16-bit slots in the 256-byte workspace
 constexpr int64_t kAmaxSharedElems = 1 << 24;
 constexpr int kAmaxSharedThreads = 256, kAmaxSharedBlocks = 512;
 __global__ void __launch_bounds__(kAmaxThreads) amax_kernel(const uint4* __restrict__ w, int64_t nvec,
-                                                            uint32_t* __restrict__ amax_bits,
-                                                            uint16_t* __restrict__ parts) {
+                                                            uint32_t* amax_bits, uint16_t* parts) {
   __shared__ uint32_t warp_max[kAmaxThreads / 32];
   pdl_launch_dependents();
   const uint32_t m = block_amax(w, nvec, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
@@ -191,9 +190,8 @@ small_scale_kernel(const uint4* __restrict__ w, int64_t nvec, float* __restrict_
 // W's start for a pass after this one (14336 x 4096, with the amax and the packing: 83.1 -> 78.0 us).
 template <bool kWide>
 __global__ void __launch_bounds__(256) rtn_codes_kernel(const uint4* __restrict__ w, int64_t groups,
-                                                        const uint32_t* __restrict__ amax, int nparts,
-                                                        float* __restrict__ global_scale,
-                                                        uint8_t* __restrict__ codes) {
+                                                        const uint32_t* amax, int nparts, float* global_scale,
+                                                        uint8_t* codes) {
   pdl_wait_primary();  // amax_kernel, when launched behind it; otherwise a no-op
   const float sg = global_scale_of(amax_of_parts(amax, nparts));
   if (blockIdx.x == 0 && threadIdx.x == 0) *global_scale = sg;

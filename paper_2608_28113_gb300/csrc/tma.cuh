@@ -113,7 +113,9 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
 }
 
 // Programmatic dependent launch: let the next kernel on the stream start its prologue,
-// and (in that kernel) wait until this one has finished and its writes are visible.
+// and (in that kernel) wait until this one has finished and its writes are visible.  A kernel
+// that waits takes what the kernel before it writes through plain pointers: __restrict__ would let the
+// compiler load it before the wait, or past the coherent caches.
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
