@@ -460,8 +460,12 @@ int hscale_output_error(const void* x_bf16, int64_t tokens, int64_t n, int64_t l
  *    accuracy (on the tensor cores: three-way bf16 splits of E and U, the six products
  *    above 2^-24 relative, fp32 accumulation).  Writes codes_out [m, n/16] and packed_out
  *    [m, n/2] (8-byte aligned) as hscale_refine_scales does.  The workspace
- *    (hscale_gptq_workspace_bytes) holds the running weights and the split operands.
- *    Blocks are taken in panels of up to 512 columns (a wider block is a panel of its own):
+ *    (hscale_gptq_workspace_bytes, 256-byte aligned) holds the running weights, m n floats, and
+ *    the split operands, max(3 panel, 12 block) bf16 for each row of W and of U, each of the three
+ *    rounded up to 256 bytes.
+ *    Blocks are taken in panels of up to 512 columns (a wider block is a panel of its own; a
+ *    workspace with 12 block bf16 a row is enough too, and then a panel has at most four blocks:
+ *    slower for blocks below 128, and the sums of each weight's updates are grouped otherwise):
  *    inside a panel each block's update reaches the panel's columns at once, and the columns
  *    right of it take the panel's update at its end, in the same order for every weight on
  *    every run (the same bits).  Everything runs on `stream`.

@@ -324,18 +324,18 @@ inline int64_t round256(int64_t bytes) { return (bytes + 255) / 256 * 256; }
 }  // namespace
 
 // running weights (fp32 m x n) and the bf16 split operands of the update: the errors
-// (m rows of three parts) and U's rows (n rows), each part as wide as the update's K; never less
-// than two buffers of 6 block per row
+// (m rows of three parts) and U's rows (n rows), each part as wide as the update's K.  Never less than
+// 12 block per row, and that is enough for a call too: its panels then have at most four blocks.
 namespace {
-inline int64_t gptq_operand_row(int64_t n, int64_t block) {
-  return std::max<int64_t>(3 * hscale::gptq_update_cols(n, block), 12 * block);
+inline int64_t gptq_least_row(int64_t block) { return 12 * block; }
+inline size_t gptq_bytes(int64_t m, int64_t n, int64_t row) {
+  return (size_t)(round256(m * n * 4) + round256(m * row * 2) + round256(n * row * 2));
 }
 }  // namespace
 
 size_t hscale_gptq_workspace_bytes(int64_t m, int64_t n, int32_t block) {
   if (m <= 0 || n <= 0 || block <= 0) return 0;
-  const int64_t row = gptq_operand_row(n, block);
-  return (size_t)(round256(m * n * 4) + round256(m * row * 2) + round256(n * row * 2));
+  return gptq_bytes(m, n, std::max(3 * hscale::gptq_update_cols(n, block), gptq_least_row(block)));
 }
 
 int hscale_gptq_hscale(const void* w_bf16, int64_t m, int64_t n, const float* U, const float* h,
@@ -351,15 +351,17 @@ int hscale_gptq_hscale(const void* w_bf16, int64_t m, int64_t n, const float* U,
     return HSCALE_ERR_NULL;
   if (!aligned(U, 16) || !aligned(h, 16) || !aligned(global_scale, 4) || !aligned(packed_out, 8))
     return HSCALE_ERR_ALIGN;
-  if (workspace == nullptr || workspace_bytes < hscale_gptq_workspace_bytes(m, n, block) || !aligned(workspace, 256))
+  if (workspace == nullptr || workspace_bytes < gptq_bytes(m, n, gptq_least_row(block)) || !aligned(workspace, 256))
     return HSCALE_ERR_WORKSPACE;
   uint8_t* base = static_cast<uint8_t*>(workspace);
-  const int64_t row = gptq_operand_row(n, block);
+  int64_t cols = hscale::gptq_update_cols(n, block);
+  if (workspace_bytes < hscale_gptq_workspace_bytes(m, n, block)) cols = std::min(cols, gptq_least_row(block) / 3);
+  const int64_t row = std::max(3 * cols, gptq_least_row(block));
   float* Wf = reinterpret_cast<float*>(base);
   uint16_t* Es = reinterpret_cast<uint16_t*>(base + round256(m * n * 4));
   uint16_t* Us = reinterpret_cast<uint16_t*>(base + round256(m * n * 4) + round256(m * row * 2));
-  return from_cuda(hscale::launch_gptq_hscale(w_bf16, m, n, U, h, global_scale, dead, block, down, up, codes_out,
-                                              packed_out, Wf, Es, Us, as_stream(stream)));
+  return from_cuda(hscale::launch_gptq_hscale(w_bf16, m, n, U, h, global_scale, dead, block, cols, down, up,
+                                              codes_out, packed_out, Wf, Es, Us, as_stream(stream)));
 }
 
 int hscale_pack_nvfp4(const void* w_bf16, int64_t m, int64_t n, const float* global_scale,

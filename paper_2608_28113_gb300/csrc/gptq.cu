@@ -597,8 +597,8 @@ int64_t gptq_update_cols(int64_t n, int64_t block) {
 // block_kernel.  Everything runs on the caller's stream, each kernel scheduled
 // while the one before it runs (programmatic dependent launch).
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
-                               const float* global_scale, const uint8_t* dead, int block, int down, int up,
-                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
+                               const float* global_scale, const uint8_t* dead, int block, int64_t cols, int down,
+                               int up, uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
                                cudaStream_t stream) {
   DeviceInfo info;
   cudaError_t err = current_device_info(&info);
@@ -609,9 +609,8 @@ cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float*
   to_fp32_kernel<<<cvt_blocks, 256, 0, stream>>>(static_cast<const uint4*>(w), m * n / 8, (uint32_t)(n / 8), dead,
                                                  reinterpret_cast<float4*>(Wf));
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
-  const int64_t step = gptq_update_cols(n, block);
-  for (int64_t c0 = 0; c0 < n; c0 += step) {
-    const int64_t K = std::min(step, n - c0), c1 = c0 + K;
+  for (int64_t c0 = 0; c0 < n; c0 += cols) {
+    const int64_t K = std::min(cols, n - c0), c1 = c0 + K;
     const bool wide = block > kPanelCols;
     // U's columns from the panel's second block on (from the next panel on for a wide block)
     const int64_t first = wide ? c1 : c0;

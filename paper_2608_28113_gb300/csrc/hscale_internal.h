@@ -115,11 +115,12 @@ cudaError_t launch_split_update(const void* a, const void* b, int64_t rows, int6
 cudaError_t launch_factor_update(const void* operand, int64_t rows, int64_t xcols, float* C, float* X, int64_t ld,
                                  int32_t order0, int32_t* info, cudaStream_t stream);
 
-// Algorithm 3's block loop.  Wf: m x n floats; Es and Us: m and n rows of 3 gptq_update_cols() bf16.
+// Algorithm 3's block loop in panels of `cols` columns (a multiple of block, or n, up to
+// gptq_update_cols()).  Wf: m x n floats; Es and Us: m and n rows of 3 cols bf16.
 int64_t gptq_update_cols(int64_t n, int64_t block);
 cudaError_t launch_gptq_hscale(const void* w, int64_t m, int64_t n, const float* U, const float* h,
-                               const float* global_scale, const uint8_t* dead, int block, int down, int up,
-                               uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
+                               const float* global_scale, const uint8_t* dead, int block, int64_t cols, int down,
+                               int up, uint8_t* codes, uint8_t* packed, float* Wf, uint16_t* Es, uint16_t* Us,
                                cudaStream_t stream);
 
 // Sticky device error flags of each translation unit (bit 0: a bounded wait ran out);

@@ -220,14 +220,14 @@ def test_factor_names_the_failed_pivot(order):
     assert np.isfinite(U).all()
 
 
-def gpu_gptq(w, U32, h32, s_g, block, down, up, dead=None):
+def gpu_gptq(w, U32, h32, s_g, block, down, up, dead=None, workspace=None):
     m, n = w.shape
     codes = torch.empty(m, n // 16, dtype=torch.uint8, device=dev())
     packed = torch.empty(m, n // 2, dtype=torch.uint8, device=dev())
     sg = torch.tensor([s_g], dtype=torch.float32, device=dev())
     dd = None if dead is None else torch.from_numpy(dead.astype(np.uint8)).to(dev())
     hs.hscale_gptq_hscale(w.to(dev()), torch.from_numpy(np.ascontiguousarray(U32)).to(dev()),
-                          torch.from_numpy(h32).to(dev()), sg, dd, block, down, up, codes, packed)
+                          torch.from_numpy(h32).to(dev()), sg, dd, block, down, up, codes, packed, workspace)
     torch.cuda.synchronize()
     return codes.cpu().numpy(), packed.cpu().numpy()
 
@@ -305,6 +305,29 @@ def test_gptq_panel_shapes(m, n, block):
     first["packed"] = ref["packed"][:, :block // 2]
     exact_outside_near_ties(codes[:, :nb], packed[:, :block // 2], first, "first block")
     assert float(np.mean(codes == ref["codes"])) >= 0.98
+    assert hs.hscale_device_error_flags() == 0
+
+
+@pytest.mark.parametrize("m,n,block", [(33, 1024, 16), (20, 1104, 48), (65, 1088, 64), (17, 1024, 128)])
+def test_gptq_workspace_of_four_blocks(m, n, block):
+    """The smallest workspace: m n floats and 12 block bf16 for each row of W and U.  The call takes it
+    in panels of at most four blocks, touches nothing beyond it and agrees with the oracle under the
+    rules above; one byte less is refused."""
+    up256 = lambda b: (b + 255) // 256 * 256
+    least = up256(4 * m * n) + up256(24 * block * m) + up256(24 * block * n)
+    assert least <= hs.hscale_gptq_workspace_bytes(m, n, block)
+    w, x, H, U32, h32, dead = layer_inputs(m, n, 600 + block, tokens=2 * n)
+    wb = bits(w)
+    s_g, _ = oracle.global_scale(wb)
+    buf = torch.full((least + 4096,), 0xEE, dtype=torch.uint8, device=dev())
+    with pytest.raises(hs.HScaleError):
+        gpu_gptq(w, U32, h32, s_g, block, 4, 4, dead=dead, workspace=buf[:least - 1])
+    codes, packed = gpu_gptq(w, U32, h32, s_g, block, 4, 4, dead=dead, workspace=buf[:least])
+    assert bool((buf[least:] == 0xEE).all())
+    ref = oracle.gptq_hscale(wb, U32.astype(np.float64), h32, s_g, block, 4, 4, dead=dead)
+    assert float(np.mean(codes == ref["codes"])) >= 0.98
+    full, _ = gpu_gptq(w, U32, h32, s_g, block, 4, 4, dead=dead)
+    assert float(np.mean(codes == full)) >= 0.98
     assert hs.hscale_device_error_flags() == 0
 
 
