@@ -227,7 +227,8 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::kBar);
   uint64_t* empty = full + kSlots;
   uint64_t* acc_full = empty + kSlots;  // four column tiles
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 4);
+  uint64_t* mma_done = acc_full + 4;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
   volatile uint32_t* failed = tmem_slot + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = (int)warp_uniform(threadIdx.x >> 5);
   const int B = args.B, outer = args.outer, gpb = B / 16, chunks = (B + 63) / 64;
@@ -241,6 +242,7 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
       mbar_init(&empty[i], 1);
     }
     for (int i = 0; i < 4; ++i) mbar_init(&acc_full[i], 1);
+    mbar_init(mma_done, 1);
     *failed = 0u;
     mbar_fence_init();
     prefetch_tensormap(&umap);
@@ -453,7 +455,7 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
     }
     const int t = warp >> 2;
     if (t < tiles) {
-      const bool done = mbar_wait(&acc_full[t], (uint32_t)b & 1u);
+      const bool done = mbar_wait_acc(&acc_full[t], (uint32_t)b & 1u);
       if (!done) *failed = 1u;
       tc_fence_after_sync();
       uint32_t p[kRows];
@@ -481,7 +483,11 @@ gptq_panel_kernel(const __grid_constant__ CUtensorMap umap, const PanelArgs args
     if (*failed) break;
   }
 
-  if (*failed && loader && lane == 0) mbar_wait(&full[slot], load_par ^ 1u);  // the slot's last load has landed
+  if (*failed) {
+    // a wait ran out: the loads (each slot's last one) and MMAs in flight finish before the CTA ends
+    if (loader) mbar_wait(&full[slot], load_par ^ 1u);
+    if (warp == 0) umma_drain(mma_done);
+  }
   __syncthreads();
   // codes and nibbles of the panel, whole rows at a time
   const int cpr = outer / 16;

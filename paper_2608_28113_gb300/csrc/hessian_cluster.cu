@@ -17,7 +17,8 @@
 // At the end the sums go through the staging area into H, row by row.
 //
 // Every wait is bounded; one that runs out sets the error flag and turns the rank's columns of the
-// tile into NaN.  The cluster leaves together.
+// tile into NaN, and the CTA's loads and MMAs in flight finish before it ends.  The cluster leaves
+// together.
 //
 // One GB300, 65536 tokens: n = 512 335 -> 73 us, 1000 667 -> 204, 2048 340 -> 247.
 #include <cooperative_groups.h>
@@ -97,7 +98,8 @@ hessian_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* ready = acc_empty + 2;  // every rank's half is in its staging area
   uint64_t* done = ready + 1;       // every rank has read this rank's staging area
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  uint64_t* mma_done = done + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
   volatile uint32_t* failed = tmem_slot + 1;
 
   cg::cluster_group cluster = cg::this_cluster();
@@ -124,6 +126,7 @@ hessian_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
     }
     mbar_init(ready, kCluster);
     mbar_init(done, kCluster);
+    mbar_init(mma_done, 1);
     *failed = 0u;
     mbar_fence_init();
     prefetch_tensormap(&amap);
@@ -178,6 +181,7 @@ hessian_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
     }
     if (!go && lane == 0) *failed = 1u;
     __syncwarp();
+    ring_drain(full, kStages, s, parity);
   } else if (warp == 1) {
     uint32_t s = 0, parity = 0, i = 0;
     bool ok = true;
@@ -221,6 +225,7 @@ hessian_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
     }
     if (!ok && lane == 0) *failed = 1u;
     __syncwarp();
+    umma_drain(mma_done);
   } else {
     // epilogue: as a source, this thread's row and 64 columns of a half; as an owner, the warp's
     // columns of the rank's share, rows 4 lane .. + 3
@@ -241,7 +246,7 @@ hessian_cluster_kernel(const __grid_constant__ CUtensorMap amap, const __grid_co
     for (int i = 0; i < rounds; ++i) {
       const uint32_t acc = (uint32_t)i & 1u;
       const bool have = i * kCluster + rank < nseg;
-      if (have && ok) ok = mbar_wait(&acc_full[acc], (uint32_t)(i >> 1) & 1u);
+      if (have && ok) ok = mbar_wait_acc(&acc_full[acc], (uint32_t)(i >> 1) & 1u);
       tc_fence_after_sync();
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf, ++turn) {

@@ -27,8 +27,8 @@
 // per row), a 4-stage ring of TMA loads (48 KB per stage).  Warp 0 issues the loads, warp 1
 // owns the tensor memory and issues the MMAs (M = 128, N = 256, K = 16 each), warps 2-9
 // read the 128 x 256 fp32 accumulator back (each warp half the columns of its 32-lane
-// quarter) and square and sum it.  Every wait is bounded; one that runs out sets the error flag and the tile's
-// partial becomes NaN.
+// quarter) and square and sum it.  Every wait is bounded; one that runs out sets the error flag and the
+// tile's partial becomes NaN, and the CTA's loads and MMAs in flight finish before it ends.
 #include <algorithm>
 #include <cuda_bf16.h>
 
@@ -172,7 +172,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
   uint64_t* empty = full + kStages;
   uint64_t* seg_full = empty + kStages;  // a segment's partial is complete
   uint64_t* seg_empty = seg_full + 1;    // the partial has been read out
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(seg_empty + 1);
+  uint64_t* mma_done = seg_empty + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
   uint32_t* failed = tmem_slot + 1;
   double* warp_sum = reinterpret_cast<double*>(smem + kStages * kStageBytes + 128);
   constexpr bool kHessian = kMode == 1 || kMode == 3;
@@ -198,6 +199,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     }
     mbar_init(seg_full, 1);
     mbar_init(seg_empty, 256);  // every epilogue thread arrives
+    mbar_init(mma_done, 1);
     *failed = 0u;
     mbar_fence_init();
     prefetch_tensormap(&xmap);
@@ -254,6 +256,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         }
       }
     }
+    ring_drain(full, kStages, s, parity);
   } else if (warp == 1) {
     // segments of kSegBlocks K blocks, each accumulated from zero
     const int nseg = (kb_total + kSegBlocks - 1) / kSegBlocks;
@@ -303,6 +306,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
     }
     if (!ok && lane == 0) atomicOr(failed, 1u);
     __syncwarp();
+    umma_drain(mma_done);
   } else {
     // epilogue warps 2-9: TMEM lane quarter warp % 4 (a warp may only touch that quarter),
     // column half (warp - 2) / 4; each thread holds one tile row's half of the partial
@@ -319,7 +323,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
       const int64_t row = (int64_t)tm * kBM + quarter * 32 + lane;
       const int64_t col0 = (int64_t)tn * kBN + cbase;
       for (int seg = 0; seg < nseg; ++seg) {
-        if (!mbar_wait(seg_full, (uint32_t)(i * nseg + seg) & 1u)) {
+        if (!mbar_wait_acc(seg_full, (uint32_t)(i * nseg + seg) & 1u)) {
           atomicOr(failed, 1u);
           alive = false;
           break;

@@ -4,6 +4,8 @@
 #pragma once
 #include <cstdint>
 
+#include "tma.cuh"
+
 namespace hscale {
 
 // ---------------------------------------------------------------- tensor memory
@@ -101,6 +103,16 @@ __device__ __forceinline__ void umma_bf16_block(uint32_t tmem_d, uint64_t adesc,
 __device__ __forceinline__ void umma_commit(uint32_t mbar_smem) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar_smem)
                : "memory");
+}
+
+// The issuing warp waits until every MMA it has issued has completed (`done`: an mbarrier of its own,
+// used once), before the CTA's shared and tensor memory may go away; after a wait that ran out nobody
+// else waits for them.
+__device__ __forceinline__ void umma_drain(uint64_t* done) {
+  if (elect_one()) umma_commit(smem_addr(done));
+  __syncwarp();
+  mbar_wait(done, 0u);
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------- tensor-memory loads

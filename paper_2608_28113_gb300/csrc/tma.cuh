@@ -9,7 +9,14 @@ namespace hscale {
 // Upper bound on polls of one mbarrier phase.  try_wait blocks for a hardware-chosen
 // interval per poll, so this is well over a second; a wait that runs out reports an
 // error instead of hanging the GPU.
-constexpr uint32_t kMbarPollLimit = 1u << 24;
+//
+// A build with HSCALE_STARVED_BLOCK = b (the failure tests') has a limit of a few milliseconds, and in
+// it mbar_wait_acc, the epilogues' wait for an accumulator, runs out at once in block b.
+#ifndef HSCALE_STARVED_BLOCK
+#define HSCALE_STARVED_BLOCK -1
+#endif
+constexpr int kStarvedBlock = HSCALE_STARVED_BLOCK;
+constexpr uint32_t kMbarPollLimit = kStarvedBlock < 0 ? 1u << 24 : 1u << 10;
 
 // Device-wide error word of this library (bit flags, sticky until read by the host).
 constexpr uint32_t kErrMbarTimeout = 1u;
@@ -57,6 +64,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return mbar_wait_bounded(bar, parity, kMbarPollLimit);
+}
+
+__device__ __forceinline__ bool mbar_wait_acc(uint64_t* bar, uint32_t parity) {
+  return (kStarvedBlock < 0 || (int)blockIdx.x != kStarvedBlock) && mbar_wait(bar, parity);
+}
+
+// The loads that a ring's producer has issued land before the CTA's shared memory may go away; after a
+// wait that ran out nobody else waits for them.  (s, parity): the producer's position, the stage it
+// would fill next and the parity of its wait for that one.  The stages before s were last filled in
+// this turn of the ring, those from s on in the turn before (or never: a fresh barrier passes).
+__device__ __forceinline__ void ring_drain(uint64_t* full, int stages, uint32_t s, uint32_t parity) {
+  for (int t = 0; t < stages; ++t) mbar_wait(&full[t], t < (int)s ? parity ^ 1u : parity);
+  __syncwarp();
 }
 
 // One lane of the (converged) warp.  The loops that issue TMA loads and MMAs run in a whole warp

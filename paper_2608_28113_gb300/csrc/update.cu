@@ -14,7 +14,7 @@
 // four 48 KB stages, 64 of K each), warp 1 owns the tensor memory and issues the MMAs, warps
 // 2-9 are the epilogue.  Two 256-column accumulators alternate, so a tile's epilogue runs
 // beside the next one's loads and MMAs.  Every wait is bounded; one that runs out sets the error
-// flag and turns the CTA's tiles into NaN.
+// flag and turns the CTA's tiles into NaN, and the CTA's loads and MMAs in flight finish before it ends.
 //
 // The factor's form (kFactor) updates the rows below diagonal block j (rows, relative to the
 // first row below it) with A = L_:j and B = [L_:j ; X_j,:^T], one operand array Bo:
@@ -149,7 +149,8 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
   uint64_t* empty = full + kStages;
   uint64_t* acc_full = empty + kStages;  // accumulator a holds a finished tile
   uint64_t* acc_empty = acc_full + 2;    // accumulator a has been read out
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* mma_done = acc_empty + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
   uint32_t* failed = tmem_slot + 1;
   const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const bool diagonal = kFactor && blockIdx.x == 0;
@@ -164,6 +165,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_empty[a], kEpiWarps * 32);
     }
+    mbar_init(mma_done, 1);
     *failed = 0u;
     mbar_fence_init();
     prefetch_tensormap(&amap);
@@ -227,6 +229,12 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     }
     if (!go && lane == 0) atomicOr(failed, 1u);
     __syncwarp();
+    if (diagonal) {
+      mbar_wait(&full[0], 0u);
+      mbar_wait(&full[1], 0u);
+    } else {
+      ring_drain(full, kStages, s, parity);
+    }
   } else if (warp == 1) {
     uint32_t s = 0, parity = 0, i = 0;  // i counts the CTA's tiles
     bool ok = true;
@@ -278,6 +286,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     }
     if (!ok && lane == 0) atomicOr(failed, 1u);
     __syncwarp();
+    umma_drain(mma_done);
   } else if (warp < 2 + kEpiWarps) {
     // epilogue: TMEM lane quarter warp % 4 (a warp may only touch that quarter), column half
     const uint32_t quarter = (uint32_t)(warp & 3), half = (uint32_t)((warp - 2) >> 2);
@@ -286,7 +295,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     if (diagonal) {
       // the next diagonal block: this thread's row, 64 columns, less the tile
       const int row = (int)quarter * 32 + lane;
-      if (mbar_wait(&full[1], 0u) && mbar_wait(&acc_full[0], 0u)) {
+      if (mbar_wait(&full[1], 0u) && mbar_wait_acc(&acc_full[0], 0u)) {
         tc_fence_after_sync();
         float* S = reinterpret_cast<float*>(smem) + row * kLd + 64 * half;  // over the operands
 #pragma unroll
@@ -333,7 +342,7 @@ update_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
             bulk_commit();
           }
         };
-        if (!mbar_wait(&acc_full[a], (i >> 1) & 1u)) {
+        if (!mbar_wait_acc(&acc_full[a], (i >> 1) & 1u)) {
           alive = false;
           break;
         }
