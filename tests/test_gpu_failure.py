@@ -107,6 +107,23 @@ def test_full_hessian_tile_of_a_starved_block(starved, monkeypatch, lead):
     assert bool(torch.isnan(got[tile]).all()) and torch.equal(got[~tile], want[~tile])
 
 
+@pytest.mark.parametrize("tokens,n", [(9000, 2000), (8192, 384), (18000, 130)])  # clusters of 2, 4 and 8
+def test_full_hessian_tile_of_a_starved_rank(starved, monkeypatch, tokens, n):
+    """The starved block is one rank of the first tile's cluster.  The others add its partial to their
+    columns, so none of the tile's values stands."""
+    x = activations(tokens, n)
+
+    def call():
+        H = torch.zeros(n, n, device="cuda")
+        hs.hscale_hessian_full_accumulate(x, H)
+        return H
+
+    got, want = both(starved, monkeypatch, call)
+    tile = torch.zeros_like(want, dtype=torch.bool)
+    tile[:128, :256] = True
+    assert bool(torch.isnan(got[tile]).all()) and torch.equal(got[~tile], want[~tile])
+
+
 def test_output_error_of_a_starved_block(starved, monkeypatch):
     x, dw2 = activations(300, 2048), activations(512, 4096)
     ws = torch.empty(hs.hscale_output_error_workspace_bytes(300, 512), dtype=torch.uint8, device="cuda")
