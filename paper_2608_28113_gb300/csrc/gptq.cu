@@ -25,25 +25,12 @@ namespace hscale {
 namespace {
 
 // ---------------------------------------------------------------- block quantizer
-__device__ __forceinline__ bool better_code(float e, int c, float be, int bc, int c0) {
-  if (e != be) return e < be;
-  const int s = c - c0, bs = bc - c0;
-  const int as = s < 0 ? -s : s, abs_ = bs < 0 ? -bs : bs;
-  return as < abs_ || (as == abs_ && s < bs);
-}
-
 // sum_j h_j (a_j - s' q_j)^2 with exact E2M1 decisions, one rounding per residual and a
 // fixed pairwise sum (relative error <= 8 * 2^-24)
 __device__ float exact_group_score(const float (&a)[16], const float (&hj)[16], uint32_t c, float sgk) {
-  const float l = e4m3_mag(c);
-  const float inv = inv_raw_of(__fmul_rn(l, sgk));
   float t[16];
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const uint32_t k = e2m1_code(a[j], inv, l, sgk);
-    const float r = __fmaf_rn(-__fmul_rn(e2m1_from_raw(k << 22), l), sgk, a[j]);
-    t[j] = __fmul_rn(hj[j], __fmul_rn(r, r));
-  }
+  for (int j = 0; j < 16; ++j) t[j] = exact_term(a[j], hj[j], c, sgk);
 #pragma unroll
   for (int step = 1; step < 16; step <<= 1)
 #pragma unroll
@@ -94,7 +81,7 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
     int bc = -1;
     for (int c = lo + q; c <= hi; c += 4) {
       const float e = exact_group_score(a, hj, (uint32_t)c, d.sgk);
-      if (bc < 0 || better_code(e, c, be, bc, c0)) {
+      if (bc < 0 || better(e, c, be, bc, c0)) {
         be = e;
         bc = c;
       }
@@ -103,7 +90,7 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
     for (int off = 1; off < 4; off <<= 1) {
       const float oe = __shfl_xor_sync(0xFFFFFFFFu, be, off);
       const int oc = __shfl_xor_sync(0xFFFFFFFFu, bc, off);
-      if (oc >= 0 && (bc < 0 || better_code(oe, oc, be, bc, c0))) {
+      if (oc >= 0 && (bc < 0 || better(oe, oc, be, bc, c0))) {
         be = oe;
         bc = oc;
       }
@@ -172,15 +159,6 @@ constexpr uint32_t kSlotBytes = 128 * 64 * 2;  // 128 columns of U, 64 of K
 constexpr int kMaxLocalBlock = kPanelCols / 2; // a larger block leaves nothing to update in the panel
 
 __device__ uint32_t g_gptq_flags = 0;
-
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int32_t c0, int32_t c1, int32_t c2,
-                                            uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_addr(bar))
-      : "memory");
-}
 
 __device__ __forceinline__ void tmem_ld_rows(uint32_t src, uint32_t (&r)[32]) { tmem_ld_32x32b_x32(src, r); }
 __device__ __forceinline__ void tmem_ld_rows(uint32_t src, uint32_t (&r)[16]) { tmem_ld_32x32b_x16(src, r); }

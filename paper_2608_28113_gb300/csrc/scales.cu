@@ -236,8 +236,8 @@ __device__ __noinline__ int warp_exact_search(const uint16_t* wg_own, const floa
 // midpoint of the grid lies between them (an exact tie among them), and those elements are
 // decided exactly with the one-FMA midpoint test of e2m1_exact_code, reading the weight back
 // from `wg` (the group's 16 bf16 values): the lower conversion gives the lower of the two
-// grid points.  A quotient below the normal range is far below the first midpoint 0.25 and
-// converts to a signed zero under both reciprocals.
+// grid points (kFromGroup: from the group's registers instead, see below).  A quotient below the normal
+// range is far below the first midpoint 0.25 and converts to a signed zero under both reciprocals.
 // Four element pairs (real-unit quotients) converted to E2M1 nibble pairs and packed into
 // one 32-bit word, pair i in byte i.
 __device__ __forceinline__ uint32_t cvt_e2m1x8(float2 y0, float2 y1, float2 y2, float2 y3) {
@@ -265,7 +265,7 @@ __device__ __forceinline__ uint32_t nonzero_nibbles(uint32_t x) {
 // 489.6 -> 491.3 us).
 template <bool kFromGroup = false>
 __device__ __forceinline__ uint2 quantize_pack(const Group& G, uint32_t c, float inv, float sgk, float pw,
-                                               const uint16_t* wg) {
+                                               const uint16_t* wg = nullptr) {
   const float ilo = __fmul_rn(inv, kBracketLo), ihi = __fmul_rn(inv, kBracketHi);
   const float2 il2 = make_float2(ilo, ilo), ih2 = make_float2(ihi, ihi);
   uint32_t lo[2], hi[2];
@@ -970,14 +970,11 @@ __global__ void __launch_bounds__(256) pack_kernel(const uint4* __restrict__ w, 
       Group G;
       unpack_group(a[u], b[u], d.pw, G);
       const uint32_t cu = c[u] < 1 ? 1u : (c[u] > kE4M3MaxCode ? kE4M3MaxCode : c[u]);
-      packed_out[gu] = quantize_pack<true>(G, cu, inv[cu], d.sgk, d.pw,
-                                     reinterpret_cast<const uint16_t*>(w) + gu * 16);
+      packed_out[gu] = quantize_pack<true>(G, cu, inv[cu], d.sgk, d.pw);
     }
   }
 }
 
-// Resident CTAs per SM of a kernel, queried once per kernel and device (the query is
-// not repeated under stream capture).
 // ---------------------------------------------------------------- 4over6 init (Algorithm 2)
 // Initial codes of Algorithm 2: for m = max|w| of the group, the E4M3 codes of m / (4 s_g)
 // and m / (6 s_g) (each as in Eq. 7), and the one whose group has the smaller plain MSE;
@@ -1002,8 +999,9 @@ __global__ void __launch_bounds__(256) fourover6_codes_kernel(const uint4* __res
   }
 }
 
-// Resident blocks per SM of kKernel at `threads` threads, queried once per device (a race
-// between threads only repeats the query: the cached value is the same either way).
+// Resident blocks per SM of kKernel at `threads` threads, queried once per device (and so not
+// under stream capture after the first call; a race between threads only repeats the query: the cached
+// value is the same either way).
 // First the kernel is given the whole shared-memory carveout.  An SM keeps the split of
 // its on-chip memory that its first resident CTA asked for, and the default split for
 // these small-shared-memory kernels leaves no room for a Hessian CTA (68 KB) beside them,

@@ -31,10 +31,6 @@ __device__ __forceinline__ void load_group_at(const uint4* wg, float pw, Group& 
   unpack_group(ld_stream_v4(wg), ld_stream_v4(wg + 1), pw, G);
 }
 
-__device__ __forceinline__ void load_group(const uint4* w, int64_t g, float pw, Group& G) {
-  load_group_at(w + 2 * g, pw, G);
-}
-
 // Per-block table of the candidate constants of every E4M3 code c (1..126), filled once
 // per CTA and stored pre-splatted for the packed arithmetic: x = y = s'^2 and
 // z = w = 1 / s' (correctly rounded), with s' = l(c) * sgk in [2^-21, 2^-2], so both are
