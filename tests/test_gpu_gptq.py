@@ -180,7 +180,7 @@ def test_factor_sizes_across_block_boundaries(n, tokens):
 @pytest.mark.parametrize("power", [-104, 90])
 def test_factor_of_a_scaled_matrix(power):
     """U of 2^power H is 2^(-power/2) U.  At these powers the pivots leave the range of the quick
-    reciprocals of the diagonal blocks (2^-100 to 2^100), so their full-range form runs; both
+    form of the diagonal blocks (2^-50 to 2^50), so their full-range form runs; both
     forms are within about 2^-22, and the factor's error grows with the condition of the damped H,
     so the bound is that of the oracle comparison above."""
     n = 300
@@ -191,6 +191,57 @@ def test_factor_of_a_scaled_matrix(power):
     assert np.all(info == 0) and np.all(infos == 0) and np.array_equal(dead, deads)
     d = np.ldexp(Us, power // 2) - U
     assert np.linalg.norm(d) <= 1e-4 * np.linalg.norm(U)
+
+
+@pytest.mark.parametrize("n", [128, 257, 640, 1000])
+def test_factor_keeps_fp32_accuracy(n):
+    """Sixteen tokens a channel: the condition of the damped H is small, so the factor's distance from
+    64 bits is that of its arithmetic: 7e-8 measured, about a unit of fp32; the bound is four times
+    that, where losing one of the products of the split operands would cost 2^-17 or more."""
+    x = calib(n, 16 * n, 900 + n)
+    H32 = oracle_H(x, n).astype(np.float32)
+    U, _, info = gpu_factor(H32)
+    Uref, _ = oracle.gptq_factor(H32.astype(np.float64))
+    assert np.all(info == 0)
+    rel = np.linalg.norm(U - Uref) / np.linalg.norm(Uref)
+    print(f"[parity] gptq factor n={n}, 16 n tokens: rel Frobenius err {rel:.2e}, worst entry "
+          f"{np.max(np.abs(U - Uref) / np.sqrt(np.outer(np.diag(Uref), np.diag(Uref)))):.2e}")
+    assert rel <= 3e-7
+
+
+def test_factor_of_the_widest_block_workload():
+    """n = 14,336 (an MLP's down projection): U^T U A v = v for the damped A, in 64 bits.  7e-7
+    measured, U's own error times the condition of A; the bound is four times that."""
+    n = 14336
+    g = torch.Generator(device=dev()).manual_seed(3)
+    x = torch.randn(2 * n, n, generator=g, device=dev())
+    H = x.T @ x
+    del x
+    U = torch.empty(n, n, device=dev())
+    info = torch.full((3,), -7, dtype=torch.int32, device=dev())
+    hs.hscale_gptq_factor(H, 0.01, U, None, info)
+    v = torch.randn(n, 4, generator=g, device=dev(), dtype=torch.float64)
+    d = torch.diagonal(H).double()
+    damp = 0.01 * d.mean()
+
+    def times(M, y, transposed=False, sym=False):  # upper triangular M, row blocks at 64 bits
+        out = torch.zeros(n, 4, dtype=torch.float64, device=dev())
+        for r in range(0, n, 2048):
+            b = torch.triu(M[r:r + 2048].double(), r)
+            if sym or not transposed:
+                out[r:r + 2048] += b @ y
+            if sym or transposed:
+                t = torch.triu(b, r + 1) if sym else b
+                out += t.T @ y[r:r + 2048]
+        return out
+
+    z = times(U, times(U, times(H, v, sym=True) + damp * v), transposed=True)
+    rel = float((z - v).norm() / v.norm())
+    print(f"[parity] gptq factor n={n}: |U^T U A v - v| / |v| {rel:.2e}")
+    assert info.cpu().tolist() == [0, 0, 0]
+    assert bool((torch.tril(U, -1) == 0).all())
+    assert rel <= 3e-6
+    assert hs.hscale_device_error_flags() == 0
 
 
 def test_factor_reports_a_matrix_that_is_not_positive_definite():
@@ -347,6 +398,57 @@ def test_gptq_rows_do_not_depend_on_the_others(m, n):
         assert np.array_equal(c, codes[r0:r1]) and np.array_equal(p, packed[r0:r1])
 
 
+@pytest.mark.parametrize("m,n,block", [
+    (300, 1024, 512),   # the update after a panel of one block
+    (200, 1536, 768),   # after a block wider than a panel
+    (300, 512, 128),    # inside a panel
+    (300, 480, 32),     # inside a panel, many blocks
+])
+def test_gptq_propagation_keeps_fp32_accuracy(m, n, block):
+    """What the propagated errors add to the weights right of them, against the same sums at 64 bits.
+    The call leaves in its workspace the running weights as each panel found them and, split, the last
+    panel's errors E, from which the running weights inside it follow.  The tensor cores' sums lose up
+    to about a unit in the last place per 16 of K, at most 2.9e-6 over 768; measured 2.4e-7 to 1.03e-6,
+    bounded by 1.6e-6.  U cut to two bf16 parts in the sums here (2.4e-6) breaks that, so the loss of
+    a product would show."""
+    w = wl.weight(m, n, 0.02, 41, dev())
+    g = torch.Generator(device=dev()).manual_seed(n)
+    U = torch.triu(torch.randn(n, n, generator=g, device=dev()), 1)
+    if n <= 512:
+        U *= 0.1  # the errors feed each other inside the panel
+    U.diagonal().copy_(1.0 + torch.rand(n, generator=g, device=dev()))
+    h, sg = torch.ones(n, device=dev()), torch.tensor([4e-5], device=dev())
+    codes = torch.empty(m, n // 16, dtype=torch.uint8, device=dev())
+    packed = torch.empty(m, n // 2, dtype=torch.uint8, device=dev())
+    ws = torch.empty(hs.hscale_gptq_workspace_bytes(m, n, block), dtype=torch.uint8, device=dev())
+    hs.hscale_gptq_hscale(w, U, h, sg, None, block, 4, 4, codes, packed, ws)
+    grid = torch.tensor([0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0], dtype=torch.float64, device=dev())
+    nib = torch.stack([packed & 15, packed >> 4], -1).view(m, n).long()
+    scale = (codes.view(torch.float8_e4m3fn).double() * sg.double()).repeat_interleave(16, 1)
+    what = torch.where((nib & 8) != 0, -1.0, 1.0).double() * grid[nib & 7] * scale
+    d = torch.diagonal(U).double()
+    if n > 512:
+        E = (w.double() - what)[:, :block] / d[:block]          # the first block's weights are w
+        got = ws[:4 * m * n].view(torch.float32).view(m, n)[:, block:].double()
+        cols = [(block, n)]
+    else:
+        at = (4 * m * n + 255) // 256 * 256
+        E = ws[at:at + 6 * m * n].view(torch.bfloat16).view(m, 3, n).double().sum(1)
+        got = (E * d + what)[:, block:]
+        cols = [(c, c + block) for c in range(block, n, block)]
+
+    def distance(V):
+        added = torch.cat([-(E[:, :a] @ V[:a, a:b]) if n <= 512 else -(E @ V[:block, a:b]) for a, b in cols], 1)
+        return float((got - w[:, block:].double() - added).norm() / added.norm())
+
+    hi = U.to(torch.bfloat16).float()
+    two_parts = hi.double() + (U - hi).to(torch.bfloat16).double()
+    rel, planted = distance(U.double()), distance(two_parts)
+    print(f"[parity] gptq propagation {m} x {n}, block {block}: {rel:.2e} from 64 bits (U in two parts {planted:.2e})")
+    assert rel <= 1.6e-6 < planted
+    assert hs.hscale_device_error_flags() == 0
+
+
 def test_gptq_zero_groups_keep_the_initial_code():
     """Groups that are all zero (dead channels) score zero under every code: the tie rule keeps
     the initial code, 1, and the nibbles are zero."""
@@ -408,10 +510,10 @@ def test_full_size_gptq_q_proj_slice():
     assert abs(err["gpu"] - err["oracle"]) <= 0.01 * err["oracle"]
 
 
-def test_gptq_look_ahead_is_deterministic_and_capturable():
-    """The block loop with the update split across two streams gives the same bytes on every
-    run, and the same bytes again when the call is captured into a CUDA graph (the second
-    stream joins the capture) and replayed."""
+def test_gptq_is_deterministic_and_capturable():
+    """The block loop, whose kernels are scheduled while the one before them runs, gives the same
+    bytes on every run, and the same bytes again when the call is captured into a CUDA graph and
+    replayed."""
     m, n, block = 256, 1024, 64
     w, x, H, U32, h32, dead = layer_inputs(m, n, 123, tokens=1024)
     wb = bits(w)

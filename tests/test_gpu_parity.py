@@ -897,7 +897,7 @@ def test_flat_schedule_matches_the_static_deal(m, n, pad, init):
     rows = torch.cat([torch.arange(8), torch.arange(m - 8, m)]).to(dev())
     wb = bits(w[rows].contiguous().cpu())
     s_ref = np.float32(sg.item())
-    first, anchor_tie = None, False
+    first, anchor_tie = None, np.zeros(1, dtype=bool)
     if init == "given":
         first = init_codes[rows].cpu().numpy()
     elif init == "4over6":
