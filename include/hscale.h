@@ -218,8 +218,8 @@ int hscale_rtn_scales(const void* w_bf16, int64_t m, int64_t n, float* global_sc
  *   runtime query) and caches it with the id of the device's context; make that first
  *   call before any stream capture.  A call in a new context of the device (after
  *   cudaDeviceReset) looks the address up again, so it is then a first call too.
- * - Every call on a device shares the array: each call clears the part it uses on its
- *   stream before use, and calls whose work overlaps on the GPU (different streams,
+ * - Every call on a device shares the array: each call writes the part it uses before it reads
+ *   it, in stream order, and calls whose work overlaps on the GPU (different streams,
  *   different threads) race with each other.  Serialise them.
  * - The scratch this work needs does not grow with m or n, so no input size is refused
  *   for lack of scratch; HSCALE_ERR_WORKSPACE would mean the work needs more than
@@ -277,7 +277,8 @@ int hscale_refine_scales(const void* w_bf16, const float* h, int64_t m, int64_t 
  * search alongside another kernel (e.g. the next input space's Hessian pass on another
  * stream).  ctas_per_sm = 0 fills every SM as hscale_refine_scales does (a search with at
  * least two 32-group units per warp then runs as one CTA of 28 warps per SM whose warps
- * share its units at run time; a smaller one as up to 7 CTAs of 4 warps per SM); k > 0
+ * share its units at run time, for ragged rows and the 2-D views of
+ * hscale_refine_scales_strided too; a smaller one as up to 7 CTAs of 4 warps per SM); k > 0
  * keeps at most k of the search's CTAs (128 threads, 72 registers each) resident per SM,
  * leaving the rest of the register file to concurrent work.  Negative values return
  * HSCALE_ERR_ARG.
@@ -441,8 +442,9 @@ int hscale_output_error(const void* x_bf16, int64_t tokens, int64_t n, int64_t l
  *    U^T U = (H + damp I)^-1, formed from the Cholesky factor of the reversed matrix and
  *    its triangular inverse (no explicit inverse of H), by the library's own kernels: a
  *    blocked Cholesky in 128-wide block columns with the triangular inverse built in the same
- *    sweep, the diagonal blocks and panels on CUDA cores and the trailing updates on the tensor
- *    cores with fp32-level accuracy (three-way bf16 splits).  info is a device int32[3]: info[0] the
+ *    sweep, the panels and the diagonal blocks' 16-wide factors on CUDA cores, the diagonal
+ *    blocks' products and the trailing updates on the tensor cores with fp32-level accuracy
+ *    (three-way bf16 splits).  info is a device int32[3]: info[0] the
  *    status of the factorization (0 = success; > 0: a pivot was not positive, the damped
  *    matrix is not positive definite, and U is unspecified), info[1] = info[2] = 0.  The
  *    workspace (hscale_gptq_factor_workspace_bytes, 256-byte aligned) holds the reversed

@@ -147,10 +147,10 @@ __global__ void __launch_bounds__(128) block_kernel(const float* __restrict__ W,
 // What bounds it: the quantizer's arithmetic and latency, then the TMA loads of U's parts
 // (96 KB per 128 columns and block of 128).  kRows is 32, or 16 when that still leaves no more
 // CTAs than SMs: half the work per CTA, and twice the lanes per group.
-// One GB300, 4096 x 4096, blocks of 128: 26-28 us a panel (53 K cycles: set-up 5,
-// quantizing 4 x 6.5, propagating 6.6 + 4.4 + 2.3, adding to the strip 3 x 0.8, write-out 1.4),
-// where the four blocks took about 130 us with a quantizer and two updates launched for each;
-// the whole call 1050 -> 628 us, 567 since its launches overlap, 554 with update.cu's last tiles
+// One GB300, 4096 x 4096, blocks of 128: 53 K cycles or 28 us a panel by clock stamps (set-up 5,
+// quantizing 4 x 6.5, propagating 6.6 + 4.4 + 2.3, adding to the strip 3 x 0.8, write-out 1.4, barriers
+// and what lies between the stamps 5), 30 us alone under a profiler; the four blocks took about 130
+// us with a quantizer and two updates launched for each; the whole call 1050 -> 628 us, 567 since its launches overlap, 554 with update.cu's last tiles
 // halved.
 constexpr int kPanelCols = 512;
 constexpr int kPanelThreads = 512;

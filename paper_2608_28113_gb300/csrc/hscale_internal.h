@@ -96,8 +96,8 @@ cudaError_t launch_hessian_cluster(int size, const CUtensorMap& amap, const CUte
                                    bool grouped, int64_t tokens, int64_t n, float* H, int64_t ld_h,
                                    cudaStream_t stream);
 
-// Algorithm 3 (GPTQ + H-Scale).  The factor's workspace (bytes) and the factor itself; U is
-// also used as scratch for the damped copy of H.
+// Algorithm 3 (GPTQ + H-Scale).  The factor's workspace (bytes) and the factor itself; U is written
+// by its last kernel only.
 int64_t gptq_factor_padded(int64_t n);
 size_t gptq_factor_workspace(int64_t n);
 cudaError_t launch_gptq_factor(const float* H, int64_t n, int64_t ld_h, float damp, float* U, uint8_t* dead,
