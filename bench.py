@@ -607,10 +607,13 @@ def step_hbm(work, ms_step: float, hbm_peak: float, peak_kind: str) -> dict:
             "note": "X once, W twice (global amax, search), codes and nibbles out, over the whole step"}
 
 
-def kernels_per_matrix(work: Work) -> int:
-    """Library kernels per matrix and step: amax and s_g (hscale_rtn_scales), the 4over6
-    codes with the two-pass init, the search."""
-    return 4 if work.init == "4over6-2pass" else 3
+def kernels_of(work: Work, M) -> int:
+    """Library kernels of one matrix and step: s_g (hscale_rtn_scales without codes: one kernel up to
+    2^20 weights; amax and s_g; from 2^24 on also the word's clearing), the 4over6 codes with the
+    two-pass init, the search."""
+    weights = M.m * M.n
+    scale = 1 if weights <= 1 << 20 else 3 if weights >= 1 << 24 else 2
+    return scale + (2 if work.init == "4over6-2pass" else 1)
 
 
 # the search kernels: one CTA per SM with a shared-memory queue (a matrix alone on the GPU),
@@ -1271,7 +1274,7 @@ def gpu_arm(args, d: Dist):
         "hessian": res["hessian"],
         "search": res["search"],
         "clocks": res["clocks"],
-        "gpu_launches": args.steps * (work.h_launches + kernels_per_matrix(work) * len(work.mats)),
+        "gpu_launches": args.steps * (work.h_launches + sum(kernels_of(work, M) for M in work.mats)),
     })
     if len(res["sweep"]) > 1:
         line["search_sweep"] = res["sweep"]
