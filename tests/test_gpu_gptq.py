@@ -209,7 +209,7 @@ def test_factor_keeps_fp32_accuracy(n):
     assert rel <= 3e-7
 
 
-def test_factor_of_the_widest_block_workload():
+def test_factor_of_a_14336_wide_layer():
     """n = 14,336 (an MLP's down projection): U^T U A v = v for the damped A, in 64 bits.  7e-7
     measured, U's own error times the condition of A; the bound is four times that."""
     n = 14336
